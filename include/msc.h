@@ -283,7 +283,7 @@ msc_status msc_saddle_arc_geometry(msc_plan_t plan, msc_stream_t stream, int64_t
  * unchanged there; the result is plan-owned until the next pass or simplification:
  *   d_alive[n_nodes] (1 = survives), d_nodeptr[n_nodes+1] / d_adj[n_adj] / d_mult[n_adj] (CSR, every
  *   arc in both rows, neighbours increasing), counts[4] (points left by index), d_log (3 uint32 per
- *   cancellation in order: upper node, lower node, round).  Host-synchronised once per round.
+ *   cancellation in order: upper node, lower node, round).  Host-synchronised every few rounds.
  *   MSC_ERR_OVERFLOW if a multiplicity exceeds 2^64 - 1; MSC_ERR_ITER_LIMIT after max_iterations
  *   rounds. */
 typedef struct msc_simplified {

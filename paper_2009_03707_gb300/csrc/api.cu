@@ -780,28 +780,14 @@ msc_status msc_simplify(msc_plan_t plan, msc_stream_t stream, const float* d_fie
     if ((st = msc::bind_device(p))) return st;
     if ((st = ensure_graph(p, s))) return st;
     if ((st = msc::run_simplify(p, d_field, threshold, s))) return st;
-    const int64_t n = p->graph_nodes;
     const int c = p->simp_cur;
-    out->n_nodes = n;
+    out->n_nodes = p->graph_nodes;
     out->n_rounds = p->simp_rounds;
     out->n_cancelled = p->simp_cancelled;
     out->n_adj = p->simp_nnz;
-    int64_t base[5] = {0, 0, 0, 0, 0};
-    for (int k = 0; k < 4; ++k) {
-        base[k + 1] = base[k] + p->counts[k];
-        out->counts[k] = 0;
-    }
-    const uint8_t* alive = static_cast<const uint8_t*>(p->simp_alive.ptr) + size_t(c) * size_t(n ? n : 1);
-    if (n) {
-        std::vector<uint8_t> h(static_cast<size_t>(n));
-        if ((st = msc::check_cuda(p, cudaMemcpyAsync(h.data(), alive, size_t(n), cudaMemcpyDeviceToHost, s), "copy out")) ||
-            (st = msc::check_cuda(p, cudaStreamSynchronize(s), "stream sync")))
-            return st;
-        for (int k = 0; k < 4; ++k)
-            for (int64_t u = base[k]; u < base[k + 1]; ++u) out->counts[k] += h[size_t(u)];
-    }
-    out->d_alive = alive;
-    out->d_nodeptr = static_cast<const int64_t*>(p->simp_ptr[c].ptr);
+    for (int k = 0; k < 4; ++k) out->counts[k] = p->simp_counts[k];
+    out->d_alive = static_cast<const uint8_t*>(p->simp_alive.ptr);
+    out->d_nodeptr = static_cast<const int64_t*>(p->simp_ptr.ptr);
     out->d_adj = static_cast<const uint32_t*>(p->simp_nbr[c].ptr);
     out->d_mult = static_cast<const uint64_t*>(p->simp_mult[c].ptr);
     out->d_log = static_cast<const uint32_t*>(p->simp_log.ptr);

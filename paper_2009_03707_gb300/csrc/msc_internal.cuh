@@ -97,10 +97,11 @@ struct Plan {
     DeviceBuffer graph_nodeptr, graph_adj, graph_mult, graph_work, graph_none;  // the 1-skeleton (graph.cu)
     DeviceBuffer geo_len, geo_off, geo_scan, geo_cells;  // cells along the saddle-extremum arcs (geometry.cu)
     DeviceBuffer ss_len, ss_off, ss_scan, ss_cells, ss_row;  // cells along the saddle-saddle arcs of count 1 (geometry.cu)
-    // simplification (simplify.cu): node cells, values, alive (two copies), keys, per-node scratch,
-    // row lengths, log positions, scan scratch, two CSRs, the log, the per-round host read-out
-    DeviceBuffer simp_cell, simp_value, simp_alive, simp_keys, simp_node, simp_len, simp_pos, simp_scan;
-    DeviceBuffer simp_ptr[2], simp_nbr[2], simp_mult[2], simp_log, simp_round;
+    // simplification (simplify.cu): alive flags, per-node and per-cancellation arrays, row lengths, log
+    // positions, scan scratch, the result's row pointers, two row pools, the log, its sort space, and the
+    // counts the host reads
+    DeviceBuffer simp_alive, simp_node, simp_len, simp_pos, simp_scan;
+    DeviceBuffer simp_ptr, simp_nbr[2], simp_mult[2], simp_log, simp_sort, simp_round;
     DeviceBuffer dp_pend, dp_in_cnt, dp_in_ptr, dp_in_idx, dp_j_off, dp_j_len, dp_pool_col, dp_pool_cnt, dp_long, dp_chunks;
 
     template <class F>
@@ -116,10 +117,9 @@ struct Plan {
                                &dp_j_len, &dp_pool_col, &dp_pool_cnt, &dp_long, &dp_chunks, &csc_colptr, &csc_row, &csc_count, &csc_work,
                                &graph_nodeptr, &graph_adj, &graph_mult, &graph_work, &graph_none,
                                &geo_len, &geo_off, &geo_scan, &geo_cells, &ss_len, &ss_off, &ss_scan, &ss_cells, &ss_row,
-                               &simp_cell, &simp_value,
-                               &simp_alive, &simp_keys, &simp_node, &simp_len, &simp_pos, &simp_scan,
-                               &simp_ptr[0], &simp_ptr[1], &simp_nbr[0], &simp_nbr[1], &simp_mult[0],
-                               &simp_mult[1], &simp_log, &simp_round};
+                               &simp_alive, &simp_node, &simp_len, &simp_pos, &simp_scan,
+                               &simp_ptr, &simp_nbr[0], &simp_nbr[1], &simp_mult[0],
+                               &simp_mult[1], &simp_log, &simp_sort, &simp_round};
         for (DeviceBuffer* b : all) f(*b);
     }
 
@@ -170,9 +170,11 @@ struct Plan {
     int64_t ss_cells_n = 0;  // cells along all saddle-saddle arcs of count 1 (geometry.cu)
     int64_t graph_nodes = 0, graph_nadj = 0;
     int64_t geo_cells_n = 0;  // cells along all arcs (geometry.cu)
-    // the last simplification (simplify.cu): which CSR copy holds it, its size, rounds, cancellations
+    // the last simplification (simplify.cu): which row pool holds its CSR, its size, rounds, cancellations,
+    // survivors per index
     int simp_cur = 0;
     int64_t simp_nnz = 0, simp_rounds = 0, simp_cancelled = 0;
+    int64_t simp_counts[4] = {0, 0, 0, 0};
     cudaEvent_t kev0 = nullptr, kev1 = nullptr;  // around the tier-0 path-count kernel
     cudaEvent_t tev0 = nullptr, tev1 = nullptr;  // around the trace kernel
     cudaEvent_t gev0 = nullptr, gev1 = nullptr;  // around the lower-star kernel

@@ -82,6 +82,21 @@ def test_anisotropic_batch_volume():
     assert np.array_equal(oracle.simplify(sk, th)["alive"], want["alive"])
 
 
+@pytest.mark.parametrize("shape,alpha,quantile", [((36, 44, 40), 2.0, 0.5), ((36, 44, 40), 2.0, 0.97), ((33, 20, 65), 3.5, 0.9)])
+def test_many_rounds_full_pools_and_long_rows(shape, alpha, quantile):
+    """Enough cancellations that the row pool fills (its rows are gathered into the other one in the
+    middle of a round), rounds beyond one batch, and rows longer than a warp."""
+    f = fields.grf(shape, alpha, seed=77)
+    sk = oracle.skeleton(f)
+    th = float(np.quantile(np.abs(sk["value"][sk["arc_u"]] - sk["value"][sk["arc_v"]]), quantile))
+    (g,) = _gpu(f, [th])
+    want = oracle.simplify(sk, th, rounds=True)
+    assert g["n_rounds"] == want["n_rounds"] > 8
+    assert np.array_equal(g["alive"], want["alive"])
+    assert np.array_equal(g["log"], np.stack([want["upper"], want["lower"], want["round"]], 1))
+    assert g["arcs"] == sorted(zip(want["arc_u"].tolist(), want["arc_v"].tolist(), want["arc_mult"].tolist()))
+
+
 def test_closed_forms():
     (g,) = _gpu(_two_wells(), [39.0])
     assert g["counts"] == [1, 0, 0, 0] and g["n_cancelled"] == 1

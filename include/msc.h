@@ -71,9 +71,11 @@ typedef struct msc_plan_s* msc_plan_t;
 typedef struct msc_opts {
     int64_t max_iterations;  /* cap on every iterative stage; 0 = 1<<20 */
     int32_t flags;           /* MSC_FLAG_* bits; other bits must be 0 */
-    int32_t path_count_tier; /* first tier of the row-wise path count: 0 = per-thread registers
-                                (default), 1 = per-warp shared-memory tables, 2 = per-CTA global
-                                tables.  Results are identical; tests use it to cover every tier. */
+    int32_t path_count_tier; /* first tier of the row-wise path count: 0 = per-thread rows, or
+                                eight lanes per row when there are few 1-saddles (default), 1 =
+                                per-warp shared-memory tables, 2 = per-CTA global tables, -1 =
+                                per-thread rows however few.  Results are identical; tests use it
+                                to cover every tier. */
     int32_t gradient_tile;   /* 0 = autotuned (the lower-star tile variant that runs fastest for the
                                 grid shape on this device, timed once per shape on the first
                                 synchronised run); 1..9 = force variant (TY,TZ,threads) =

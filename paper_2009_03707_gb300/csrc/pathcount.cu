@@ -15,7 +15,10 @@
 // that can hold it, to keep as many rows in flight as possible:
 //   tier 0  a row per lane, frontier (<= 8) and D* row (<= 16) hash tables in shared memory,
 //           32-bit counts; each frontier step is spread over the warp item by item;
-//   tier 1  one warp per row, 256-slot hash tables in shared memory;
+//   tier 0b eight lanes per row, frontier (<= 48) and D* row (<= 112) tables in shared memory,
+//           32-bit counts: the rows that outgrow tier 0 (about 1 %), or all of them when there
+//           are too few to fill the device's lanes;
+//   tier 1  one warp per row, 256-slot hash tables in shared memory, uint64 counts;
 //   tier 2+ one CTA per row, hash tables in global memory, grown until the row fits.
 // A row that overflows its worker is deferred, intact, to the next tier.  Finished rows are
 // sorted by column and appended to a staging buffer; a scan of the row lengths and one gather
@@ -29,12 +32,19 @@ namespace {
 constexpr uint32_t EMPTY = 0xFFFFFFFFu;
 constexpr int T0_WARPS = 8;
 constexpr int T0_THREADS = T0_WARPS * 32;
-// tier 0: frontier and D* table slots per row (powers of two); tier 0b: the same kernel with
-// larger tables for the few rows that outgrow tier 0 (more shared memory per row, so fewer rows
-// in flight -- which only the deferred rows pay for)
+// tier 0: frontier and D* table slots per row (powers of two)
 constexpr int T0_F = 8, T0_LF = 3, T0_D = 16, T0_LD = 4;
-constexpr int T0B_F = 16, T0B_LF = 4, T0B_D = 32, T0B_LD = 5;
 constexpr int T0_OUT_CHUNK = 1024;  // staging slots a warp takes at a time
+// tier 0b: lanes per row, table slots and the entries they may hold
+constexpr int TG_LANES = 8, TG_ROWS = 32 / TG_LANES;
+constexpr int TG_F = 64, TG_LF = 6, TG_FMAX = 48, TG_D = 128, TG_LD = 7, TG_DMAX = 112;
+constexpr int TG_WARPS = 8, TG_THREADS = TG_WARPS * 32;
+constexpr int TG_OUT_CHUNK = 256;
+// Up to this many 1-saddles start in tier 0b: tier 0's steps are longer (it packs 32 rows on a warp),
+// which pays when there are rows enough for every warp.  Path-count stage, tier 0 first against tier 0b
+// first: 36 thousand 1-saddles 0.176 and 0.112 ms, 467 thousand 0.267 and 0.420 ms; the lines through
+// these cross near 160 thousand.
+constexpr int64_t GROUP_FIRST = 128 * 1024;
 constexpr int T1_WARPS = 4;
 constexpr int T1_HASH = 256;  // slots per table (power of two)
 constexpr int T1_LIST = T1_HASH / 2;
@@ -410,6 +420,202 @@ __global__ void __launch_bounds__(T0_THREADS) rows_thread(PcArgs args, u64* next
 }
 
 // ---------------------------------------------------------------------------------------
+// tier 0b: eight lanes per row
+// ---------------------------------------------------------------------------------------
+// The rows that outgrow tier 0 are few and deep, so what counts is how long one step of one row
+// takes.  A group of eight lanes owns a row; its frontier entries are expanded eight at a time, each
+// by one lane, and the slots claimed in the next table are listed as they are claimed, so a step
+// reads and clears only what is used.  The four groups of a warp step together (their loops run as
+// long as the longest, so the warp does not diverge).  Tables hold 32-bit counts; a row whose table
+// fills up or whose counts wrap goes on to the warp tier.
+// Against a lane per row with 16- and 32-slot tables, where a warp took 32 such rows at once and
+// a step was ten rounds of gathers: 202 -> 62 us on a 61 x 75 x 49 GRF, 256 -> 163 on the 256^3 GRF,
+// 345 -> 171 on a 203 x 256 x 178 8-bit field; and the warp tier, which gets hardly any rows now,
+// 60-107 -> 7 us.
+struct GroupRow {
+    uint32_t fk[2][TG_F], fv[2][TG_F];  // frontier tables (current and next): key, count
+    uint32_t dk[TG_D], dv[TG_D];        // D* row
+    uint8_t fl[2][TG_F], dl[TG_D];      // the slots in use, in claim order
+    int fn[2], dn;                      // and how many
+};
+
+// Adds val to key's entry in one of the row's tables (lanes of the group may add at once); false if
+// the table is full or the count wraps.
+__device__ __forceinline__ bool group_add(uint32_t* K, uint32_t* V, uint8_t* list, int* n, int limit, int lg, uint32_t key,
+                                          uint32_t val) {
+    const uint32_t mask = (1u << lg) - 1u;
+    uint32_t h = (key * 2654435761u) >> (32 - lg);
+#pragma unroll 1
+    for (uint32_t p = 0; p <= mask; ++p, h = (h + 1) & mask) {
+        uint32_t k = *reinterpret_cast<volatile uint32_t*>(&K[h]);
+        if (k == EMPTY) {
+            k = atomicCAS(&K[h], EMPTY, key);
+            if (k == EMPTY) {
+                const int at = atomicAdd(n, 1);
+                if (at >= limit) return false;  // the row is deferred and its tables scrubbed
+                list[at] = uint8_t(h);
+                k = key;
+            }
+        }
+        if (k == key) {
+            const uint32_t old = atomicAdd(&V[h], val);
+            return old + val >= old;
+        }
+    }
+    return false;
+}
+
+__device__ __forceinline__ void group_scrub(GroupRow& t, int r) {
+    for (int j = r; j < TG_F; j += TG_LANES) {
+        t.fk[0][j] = t.fk[1][j] = EMPTY;
+        t.fv[0][j] = t.fv[1][j] = 0;
+    }
+    for (int j = r; j < TG_D; j += TG_LANES) {
+        t.dk[j] = EMPTY;
+        t.dv[j] = 0;
+    }
+    if (r == 0) t.fn[0] = t.fn[1] = t.dn = 0;
+}
+
+__global__ void __launch_bounds__(TG_THREADS) rows_group(PcArgs args, u64* next_row) {
+    PcArgs a = args;
+    if (!resolve(a)) return;
+    extern __shared__ __align__(16) unsigned char tg_raw[];
+    const int lane = threadIdx.x & 31, g = lane / TG_LANES, r = lane % TG_LANES;
+    GroupRow& t = reinterpret_cast<GroupRow*>(tg_raw)[(threadIdx.x >> 5) * TG_ROWS + g];
+    const uint32_t lead = 0x01010101u;  // the first lane of every group
+    group_scrub(t, r);
+    __syncwarp();
+    int64_t s = -1;  // the group's row (-1: none)
+    int c = 0;       // which frontier table is current (warp-uniform)
+    bool exhausted = false;
+    u64 iter = 0, entries = 0, it_max = 0, en_sum = 0, mx_all = 0;
+    u64 out_next = 0, out_end = 0;  // the warp's staging chunk
+    while (true) {
+        const uint32_t want = __ballot_sync(0xFFFFFFFFu, s < 0 && !exhausted) & lead;
+        if (want) {
+            u64 first = 0;
+            if (lane == 0) first = atomicAdd(next_row, (u64)__popc(want));
+            first = __shfl_sync(0xFFFFFFFFu, first, 0);
+            if (s < 0 && !exhausted) {
+                const u64 mine = first + u64(__popc(want & ((1u << (g * TG_LANES)) - 1u)));
+                if (mine < (u64)a.nrows) {  // a new row starts from A[s,:] and D[s,:]
+                    s = row_of(a, int64_t(mine));
+                    iter = entries = 0;
+                    if (r < 4) {
+                        const uint32_t kind = trace_kind(a.kinds[s], r), dst = a.tgt[4 * s + r];
+                        if (kind == 1) group_add(t.fk[c], t.fv[c], t.fl[c], &t.fn[c], TG_FMAX, TG_LF, dst, 1);
+                        if (kind == 2) group_add(t.dk, t.dv, t.dl, &t.dn, TG_DMAX, TG_LD, dst, 1);
+                    }
+                } else {
+                    exhausted = true;
+                }
+            }
+        }
+        if (!__any_sync(0xFFFFFFFFu, s >= 0)) break;
+        __syncwarp();
+        // one frontier step of every row
+        const int n = s >= 0 ? t.fn[c] : 0;
+        bool expand = true;
+        if (n && int64_t(++iter) > a.max_iter) {
+            if (r == 0) atomicOr(a.status, ST_ITER);  // the row is cut short; the result is void anyway
+            expand = false;
+        }
+        entries += u64(n);
+        bool ok = true;
+        for (int i = r; __any_sync(0xFFFFFFFFu, i < n); i += TG_LANES) {
+            if (i >= n) continue;
+            const int slot = t.fl[c][i];
+            const uint32_t key = t.fk[c][slot], cnt = t.fv[c][slot];
+            t.fk[c][slot] = EMPTY;
+            t.fv[c][slot] = 0;
+            if (!expand) continue;
+            const int64_t src = a.n1 + int64_t(key);
+            const uint32_t kj = a.kinds[src];
+            const uint4 q = trace_of(a, src);
+            const uint32_t tq[4] = {q.x, q.y, q.z, q.w};
+#pragma unroll
+            for (int k = 0; k < 4; ++k) {
+                const uint32_t kind = trace_kind(kj, k);
+                if (!kind) continue;
+                const bool j = kind == 1;
+                ok &= group_add(j ? t.fk[c ^ 1] : t.dk, j ? t.fv[c ^ 1] : t.dv, j ? t.fl[c ^ 1] : t.dl,
+                                j ? &t.fn[c ^ 1] : &t.dn, j ? TG_FMAX : TG_DMAX, j ? TG_LF : TG_LD, tq[k], cnt);
+            }
+        }
+        const uint32_t bad = __ballot_sync(0xFFFFFFFFu, !ok);
+        __syncwarp();
+        if (r == 0) t.fn[c] = 0;
+        c ^= 1;
+        const bool defer = s >= 0 && ((bad >> (g * TG_LANES)) & ((1u << TG_LANES) - 1u));
+        const bool done = s >= 0 && !defer && t.fn[c] == 0;
+        // finished rows, each entry at its rank (rows come out sorted by column)
+        const int nd = done ? t.dn : 0;
+        u64 base = 0;
+        unsigned nout = 0;
+        for (int k = 0; k < TG_ROWS; ++k) {
+            const int len = __shfl_sync(0xFFFFFFFFu, nd, k * TG_LANES);
+            if (k < g) base += u64(len);
+            nout += unsigned(len);
+        }
+        if (nout) {
+            if (u64(nout) > out_end - out_next) {
+                const u64 ch = max(u64(nout), u64(TG_OUT_CHUNK));
+                u64 b = 0;
+                if (lane == 0) b = atomicAdd(a.out_cursor, ch);
+                out_next = __shfl_sync(0xFFFFFFFFu, b, 0);
+                out_end = out_next + ch;
+            }
+            base += out_next;
+            out_next += u64(nout);
+            for (int i = r; i < nd; i += TG_LANES) {
+                const uint32_t key = t.dk[t.dl[i]], val = t.dv[t.dl[i]];
+                int rank = 0;
+                for (int e = 0; e < nd; ++e) rank += t.dk[t.dl[e]] < key;
+                const u64 dst = base + u64(rank);
+                if (dst < a.out_cap) {
+                    a.out_col[dst] = key;
+                    a.out_cnt[dst] = val;
+                } else {
+                    atomicOr(a.status, ST_RETRY);  // staging too small: the host grows it and reruns
+                }
+                mx_all = max(mx_all, (u64)val);
+            }
+            __syncwarp();
+            for (int i = r; i < nd; i += TG_LANES) {
+                t.dk[t.dl[i]] = EMPTY;
+                t.dv[t.dl[i]] = 0;
+            }
+            __syncwarp();
+        }
+        if (done) {
+            if (r == 0) {
+                a.row_start[s] = nd ? int64_t(base) : 0;
+                a.row_len[s] = uint32_t(nd);
+                t.dn = 0;
+            }
+            it_max = max(it_max, iter);
+            if (r == 0) en_sum += entries;
+            s = -1;
+        }
+        if (defer) {
+            if (r == 0) a.deferred[atomicAdd(a.deferred_count, 1ull)] = uint32_t(s);
+            group_scrub(t, r);
+            s = -1;
+        }
+        __syncwarp();
+    }
+    mx_all = warp_max(mx_all);
+    it_max = warp_max(it_max);
+    en_sum = warp_sum(en_sum);
+    if (lane == 0) {
+        if (mx_all) atomicMax(a.max_count, mx_all);
+        if (it_max) atomicMax(a.n_iter, it_max);
+        if (en_sum) atomicAdd(a.n_entries, en_sum);
+    }
+}
+
+// ---------------------------------------------------------------------------------------
 // tiers 1 and 2+: hash tables shared by a group of G threads
 // ---------------------------------------------------------------------------------------
 struct Tables {
@@ -699,7 +905,7 @@ __global__ void gather_rows(const unsigned long long* n1_dev, int64_t cap, const
 
 // Counter slots in Summary::pc.
 enum { C_CURSOR = PC_CURSOR, C_MAX = PC_MAX, C_ITER = PC_ITER, C_ENTRIES = PC_ENTRIES, C_DEFER0 = PC_DEFER0,
-       C_DEFER1 = PC_DEFER1, C_NEXT = PC_NEXT, C_DEFER2 = PC_DEFER2, C_DEFER3 = PC_DEFER3 };
+       C_DEFER1 = PC_DEFER1, C_NEXT = PC_NEXT, C_DEFER2 = PC_DEFER2, C_DEFER3 = PC_DEFER3, C_NEXT_GROUP = PC_NEXT_GROUP, C_NEXT_WARP = PC_NEXT_WARP };
 
 }  // namespace
 
@@ -731,7 +937,9 @@ msc_status run_path_count(Plan* p, cudaStream_t s) {
             if ((st = ensure(p, p->pc_cnt, sizeof(u64) * cap))) return st;
             if ((st = ensure(p, p->dstar_col, sizeof(uint32_t) * cap))) return st;
             if ((st = ensure(p, p->dstar_count, sizeof(u64) * cap))) return st;
-            if ((st = check_cuda(p, cudaMemsetAsync(ctr, 0, sizeof(u64) * PC_SLOTS, s), "memset counters"))) return st;
+            // a captured pass starts from a cleared summary, and its path count runs once
+            if (!cap_mode && (st = check_cuda(p, cudaMemsetAsync(ctr, 0, sizeof(u64) * PC_SLOTS, s), "memset counters")))
+                return st;
             if ((st = run_junction_dp(p, s, pool, cap))) return st;
             if (!cap_mode) {
                 if ((st = read_summary(p, s))) return st;
@@ -775,25 +983,24 @@ msc_status run_path_count(Plan* p, cudaStream_t s) {
     // a row whose counts pass 255 then goes on to tier 0b, which keeps 32-bit counts.
     const bool pack = njcap < int64_t(0xFFFFFF) && n2cap < int64_t(0xFFFFFF);
     const size_t t0_smem = (pack ? sizeof(T0Warp<T0_F, T0_D, true>) : sizeof(T0Warp<T0_F, T0_D, false>)) * T0_WARPS;
-    const size_t t0b_smem = sizeof(T0Warp<T0B_F, T0B_D, false>) * T0_WARPS;
+    const size_t tg_smem = sizeof(GroupRow) * TG_ROWS * TG_WARPS;
     auto* k0 = pack ? rows_thread<T0_F, T0_LF, T0_D, T0_LD, true> : rows_thread<T0_F, T0_LF, T0_D, T0_LD, false>;
-    auto* k0b = rows_thread<T0B_F, T0B_LF, T0B_D, T0B_LD, false>;
     if ((st = check_cuda(p, cudaFuncSetAttribute(k0, cudaFuncAttributeMaxDynamicSharedMemorySize, int(t0_smem)),
                          "cudaFuncSetAttribute(rows_thread)")) ||
-        (st = check_cuda(p, cudaFuncSetAttribute(k0b, cudaFuncAttributeMaxDynamicSharedMemorySize, int(t0b_smem)),
-                         "cudaFuncSetAttribute(rows_thread)")))
+        (st = check_cuda(p, cudaFuncSetAttribute(rows_group, cudaFuncAttributeMaxDynamicSharedMemorySize, int(tg_smem)),
+                         "cudaFuncSetAttribute(rows_group)")))
         return st;
     int per_sm = 0, per_sm_b = 0;
     cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k0, T0_THREADS, t0_smem);
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm_b, k0b, T0_THREADS, t0b_smem);
+    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm_b, rows_group, TG_THREADS, tg_smem);
     const int t0_grid = int(std::max<int64_t>(
         1, std::min<int64_t>((n1cap + T0_THREADS - 1) / T0_THREADS, int64_t(std::max(1, per_sm)) * p->num_sms)));
-    const int t0b_grid = int(std::max<int64_t>(
-        1, std::min<int64_t>((n1cap + T0_THREADS - 1) / T0_THREADS, int64_t(std::max(1, per_sm_b)) * p->num_sms)));
+    const int tg_grid = int(std::max<int64_t>(
+        1, std::min<int64_t>((n1cap + TG_ROWS * TG_WARPS - 1) / (TG_ROWS * TG_WARPS), int64_t(std::max(1, per_sm_b)) * p->num_sms)));
     // staging capacity, including what tier-0 warps may leave unused at the end of their chunks;
     // a synchronised run grows it and reruns the stage on overflow, a replayed graph asks for a rerun
     const uint64_t slack = uint64_t(t0_grid) * T0_WARPS * (T0_OUT_CHUNK + 32 * T0_D) +
-                           uint64_t(t0b_grid) * T0_WARPS * (T0_OUT_CHUNK + 32 * T0B_D);
+                           uint64_t(tg_grid) * TG_WARPS * (TG_OUT_CHUNK + TG_ROWS * TG_D);
     uint64_t cap = cap_mode ? uint64_t(p->caps.staging)
                             : uint64_t(std::max<int64_t>(p->dstar_nnz + p->dstar_nnz / 4, 8 * n1cap + 1024)) + slack;
     // a row never needs more slots than 2 x max(junctions, 2-saddles)
@@ -804,7 +1011,8 @@ msc_status run_path_count(Plan* p, cudaStream_t s) {
         if ((st = ensure(p, p->pc_cnt, sizeof(u64) * cap))) return st;
         if ((st = ensure(p, p->dstar_col, sizeof(uint32_t) * cap))) return st;
         if ((st = ensure(p, p->dstar_count, sizeof(u64) * cap))) return st;
-        if ((st = check_cuda(p, cudaMemsetAsync(ctr, 0, sizeof(u64) * PC_SLOTS, s), "memset counters"))) return st;
+        if (!cap_mode && (st = check_cuda(p, cudaMemsetAsync(ctr, 0, sizeof(u64) * PC_SLOTS, s), "memset counters")))
+            return st;
         PcArgs a{};
         a.n1_dev = &p->dsum()->counts[1];
         a.nj_dev = &p->dsum()->n_junctions;
@@ -832,17 +1040,18 @@ msc_status run_path_count(Plan* p, cudaStream_t s) {
             a.deferred_count = defer_ctr;
             a.retry_on_defer = last && cap_mode;
             msc_status e;
-            if (tier != 2 && (e = check_cuda(p, cudaMemsetAsync(ctr + C_NEXT, 0, sizeof(u64), s), "memset"))) return e;
             if (tier == 0) {
                 record_event(p, p->kev0, s);
                 k0<<<t0_grid, T0_THREADS, t0_smem, s>>>(a, ctr + C_NEXT);
                 record_event(p, p->kev1, s);
                 launched(p);
             } else if (tier == 3) {
-                k0b<<<t0b_grid, T0_THREADS, t0b_smem, s>>>(a, ctr + C_NEXT);
+                if (!rows) record_event(p, p->kev0, s);  // it is the first tier
+                rows_group<<<tg_grid, TG_THREADS, tg_smem, s>>>(a, ctr + C_NEXT_GROUP);
+                if (!rows) record_event(p, p->kev1, s);
                 launched(p);
             } else if (tier == 1) {
-                rows_warp<<<std::max(1, p->num_sms) * 8, T1_WARPS * 32, 0, s>>>(a, ctr + C_NEXT);
+                rows_warp<<<std::max(1, p->num_sms) * 8, T1_WARPS * 32, 0, s>>>(a, ctr + C_NEXT_WARP);
                 launched(p);
             } else {
                 const int cap_t = 1 << lg;
@@ -871,8 +1080,12 @@ msc_status run_path_count(Plan* p, cudaStream_t s) {
         int left_list = 1;
         u64* left_ctr = ctr + C_DEFER2;
         if (first_tier == 0) {
-            if ((st = launch(0, nullptr, all_rows, lists[0], ctr + C_DEFER0, 0, false))) return st;
-            if ((st = launch(3, lists[0], ctr + C_DEFER0, lists[1], ctr + C_DEFER1, 0, false))) return st;
+            if (n1cap > GROUP_FIRST || p->opts.path_count_tier < 0) {
+                if ((st = launch(0, nullptr, all_rows, lists[0], ctr + C_DEFER0, 0, false))) return st;
+                if ((st = launch(3, lists[0], ctr + C_DEFER0, lists[1], ctr + C_DEFER1, 0, false))) return st;
+            } else if ((st = launch(3, nullptr, all_rows, lists[1], ctr + C_DEFER1, 0, false))) {
+                return st;
+            }
             if ((st = launch(1, lists[1], ctr + C_DEFER1, lists[0], ctr + C_DEFER3, 0, false))) return st;
             if ((st = launch(2, lists[0], ctr + C_DEFER3, lists[1], ctr + C_DEFER2, lg, true))) return st;
         } else if (first_tier == 1) {

@@ -374,7 +374,8 @@ msc_status finish_replay(Plan* p, cudaStream_t s) {
     p->stage_recorded = 0x3F;
     p->stats.n_launches = p->graph_static_launches + p->loop_body_launches[0] * int64_t(p->hsum->jump_rounds) +
                           p->loop_body_launches[1] * int64_t(p->hsum->sweep_iters) +
-                          p->loop_body_launches[2] * int64_t(p->hsum->dp_iters);
+                          p->loop_body_launches[2] * int64_t(p->hsum->dp_iters) +
+                          p->loop_body_launches[3] * int64_t(p->hsum->push_iters);
     p->have_gradient = p->have_critical = p->have_extremum = p->have_reach = true;
     p->have_junctions = p->have_trace = p->have_dstar = true;
     ++p->graph_replays;

@@ -64,7 +64,9 @@ struct Summary {
     uint32_t pad;
     uint32_t jump_flag[2];            // pointer jumping's own "changed" flag and continue decision: that
                                       // stage runs beside the reachability loop in a replayed pass
-    uint32_t pad3[2];
+    uint32_t push_count[5];           // reachability: the new cells of the pushed levels in hand (reach.cu)
+    uint32_t push_cursor;             // reachability: places taken in the queue they start from
+    unsigned long long push_iters;    // iterations of the pushed-level loop
 };
 
 // ---- the plan ----------------------------------------------------------------------------
@@ -88,7 +90,7 @@ struct Plan {
     DeviceBuffer words, status, crit_bits, crit_prefix, scan_sums;
     DeviceBuffer cells[4];
     DeviceBuffer vmin, cmax, min_arcs, max_arcs, ext_lab_v, ext_lab_c;
-    DeviceBuffer visited, reach_tmp, reach_masks, reach_qdown, reach_stamp, node_info;
+    DeviceBuffer visited, reach_tmp, reach_masks, reach_qdown, reach_stamp, reach_queue, node_info;
     DeviceBuffer junc_bits, junc_prefix, junc_cells;
     DeviceBuffer trace, trace_kinds, minor_rowcnt, minor_scan, minor_rowptr[4], minor_col[4], minor_mult[4];
     DeviceBuffer pc_rowstart, pc_rowlen, pc_big, pc_col, pc_cnt, pc_gk, pc_gv, pc_gocc;
@@ -108,7 +110,7 @@ struct Plan {
     void for_each_buffer(F&& f) {
         DeviceBuffer* all[] = {&words, &status, &crit_bits, &crit_prefix, &scan_sums, &cells[0], &cells[1], &cells[2],
                                &cells[3], &vmin, &cmax, &min_arcs, &max_arcs, &ext_lab_v, &ext_lab_c, &visited, &reach_tmp, &reach_masks,
-                               &reach_qdown, &reach_stamp, &node_info, &junc_bits, &junc_prefix, &junc_cells, &trace, &trace_kinds,
+                               &reach_qdown, &reach_stamp, &reach_queue, &node_info, &junc_bits, &junc_prefix, &junc_cells, &trace, &trace_kinds,
                                &minor_rowcnt, &minor_scan, &minor_rowptr[0], &minor_rowptr[1], &minor_rowptr[2],
                                &minor_rowptr[3], &minor_col[0], &minor_col[1], &minor_col[2], &minor_col[3],
                                &minor_mult[0], &minor_mult[1], &minor_mult[2], &minor_mult[3], &pc_rowstart, &pc_rowlen,
@@ -144,13 +146,16 @@ struct Plan {
     cudaGraphExec_t graph_exec = nullptr;
     const float* graph_field = nullptr;
     int64_t graph_static_launches = 0;  // kernels per replay outside the loops
-    int64_t loop_body_launches[3] = {0, 0, 0};  // per iteration: pointer jumping, reachability, DP waves
+    int64_t loop_body_launches[4] = {0, 0, 0, 0};  // per iteration: pointer jumping, reachability sweeps, DP waves, pushes
     Summary* hsum = nullptr;          // pinned host mirror of the summary
     cudaEvent_t stage_ev[12] = {};    // start and end of stages 0..5 (read by msc_get_stats)
     uint32_t stage_recorded = 0;      // stages whose two events belong to the same pass
     bool caps_ready = false;          // a synchronised run has measured the sizes
     int64_t graph_replays = 0;
     int64_t capture_epoch = 0;        // bumped whenever the plan's graph is captured or dropped
+    int tail_cluster = 0;             // blocks of the reachability's last-levels cluster (0: not asked yet)
+    int64_t reach_iters = 1;          // sweep iterations of the last synchronised pass (two sweeps each)
+    bool reach_sweeps_only = false;   // a level outgrew the push queue on this plan
     int grad_variant = -1;            // gradient tile variant (-1: not tuned yet)
 
     int64_t counts[4] = {0, 0, 0, 0};

@@ -18,14 +18,28 @@
 //    per node over the whole grid.  One loop iteration is two sweeps (A -> B, B -> A, so the
 //    set always ends in A) and a one-thread decision kernel; the loop is a conditional WHILE node
 //    when the pipeline runs as a graph, so no level needs a host round trip.
+//  * A sweep costs the same however few cells it adds, and most levels add few (512^3 blob field:
+//    153 levels, 7.9 M new cells at level 1, 1.4 M at level 11, then 3 % fewer each; 256^3 GRF: 14
+//    levels, 8.4 M at level 2, 0.1 M at level 6).  So the sweeps stop once a level is sparse, the
+//    cells of that last level become a queue, and the other levels are pushed: each new cell's
+//    out-edges set their targets' bits and append the targets that were not set.  The level sets are
+//    the same.  Large grids push with the whole device while a level is large; the last levels --
+//    and on a small grid all of them -- run in one kernel of one thread-block cluster, whose
+//    hardware barrier between levels costs far less than a kernel boundary.
+//    Reachability stage: 512^3 blobs 15.9 -> 4.9 ms, 256^3 GRF 0.395 -> 0.299, 61 x 75 x 49 GRF 0.102 ->
+//    0.072, 32^3 lattice (19 levels) 0.127 -> 0.072.
 //
 // Sec. 3.3 / Sec. 3.5 "Gradient path counting": a junction is a reachable 1-cell that is not a
 // 1-saddle and has out-degree > 1.  One warp per bitmap word (a lane per 1-cell) evaluates the
 // out-edges of each reachable cell, marks junctions, and records each node's successor for the
 // path tracer.  Junctions are stream-compacted in cell-id order (scan.cuh), which also gives
 // O(1) ranks for the minor's matrix indices.
+#include <cooperative_groups.h>
+
 #include "dag.cuh"
 #include "scan.cuh"
+
+namespace cg = cooperative_groups;
 
 namespace msc {
 
@@ -177,7 +191,7 @@ __global__ void __launch_bounds__(THREADS) reach_init(Geom g, const uint32_t* __
 }
 
 template <int A>
-__device__ __forceinline__ bool sweep_word(const Rows& r, const uint4* __restrict__ masks,
+__device__ __forceinline__ uint32_t sweep_word(const Rows& r, const uint4* __restrict__ masks,
                                            const uint32_t* __restrict__ Rin, uint32_t* __restrict__ Rout) {
     constexpr int B1 = A == 0 ? 1 : 0, B2 = A == 2 ? 1 : 2;
     const int i = r.edge<A>(0, 0);
@@ -188,12 +202,12 @@ __device__ __forceinline__ bool sweep_word(const Rows& r, const uint4* __restric
         add = pull<A, B1, -1>(m.x & ~cur, Rin, r) | pull<A, B1, 1>(m.y & ~cur, Rin, r) |
               pull<A, B2, -1>(m.z & ~cur, Rin, r) | pull<A, B2, 1>(m.w & ~cur, Rin, r);
     Rout[i] = cur | add;
-    return add != 0;
+    return __popc(add);
 }
 
 // One level: Rout = Rin | cells whose partner quad has another facet in Rin.  A thread takes one
 // vertex-row word at a time for all three axes (one neighbourhood check, three independent chains
-// of loads).  Sets *changed if any word grew.
+// of loads).  Adds the number of new cells to *added.
 // Rows (y, z) are stamped with 1 + the last sweep that changed them (1: the start).  A cell's
 // predecessors lie within one step in y and z, so a row none of whose 3 x 3 neighbour rows changed
 // in the previous sweep cannot change now; it is skipped, Rout included: that buffer already
@@ -202,10 +216,11 @@ __device__ __forceinline__ bool sweep_word(const Rows& r, const uint4* __restric
 __global__ void __launch_bounds__(THREADS, 4) reach_sweep(Geom g, const uint4* __restrict__ masks,
                                                        const uint32_t* __restrict__ Rin, uint32_t* __restrict__ Rout,
                                                        uint32_t* __restrict__ stamp, const Summary* __restrict__ sum,
-                                                       int parity, uint32_t* __restrict__ changed) {
+                                                       int parity, uint32_t* __restrict__ added) {
+    if (!sum->loop_flag[3]) return;  // a replayed pass has swept enough
     const int64_t nrw = int64_t(g.nz) * g.ny * g.W;
     const uint32_t k = 2u * uint32_t(sum->sweep_iters) + 1u + uint32_t(parity);  // this sweep
-    bool grew = false;
+    uint32_t grew = 0;
     // grid-stride over the row words (a few tiles of THREADS words per CTA): a sweep in which few
     // rows are near a front then costs fewer CTA launches for the rest
     for (int64_t t = int64_t(blockIdx.x) * THREADS + threadIdx.x; t < nrw; t += int64_t(gridDim.x) * THREADS) {
@@ -217,36 +232,350 @@ __global__ void __launch_bounds__(THREADS, 4) reach_sweep(Geom g, const uint4* _
                 if (y >= 0 && y < g.ny && z >= 0 && z < g.nz) recent = max(recent, stamp[int64_t(z) * g.ny + y]);
             }
         if (recent >= k) {
-            const bool g0 = sweep_word<0>(r, masks, Rin, Rout);
-            const bool g1 = sweep_word<1>(r, masks, Rin, Rout);
-            const bool g2 = sweep_word<2>(r, masks, Rin, Rout);
-            if (g0 || g1 || g2) {
-                stamp[int64_t(r.z) * g.ny + r.y] = k + 1;
-                grew = true;
-            }
+            const uint32_t n = sweep_word<0>(r, masks, Rin, Rout) + sweep_word<1>(r, masks, Rin, Rout) +
+                               sweep_word<2>(r, masks, Rin, Rout);
+            if (n) stamp[int64_t(r.z) * g.ny + r.y] = k + 1;
+            grew += n;
         }
     }
-    if (__syncthreads_or(grew) && threadIdx.x == 0) *changed = 1u;
+    grew = __reduce_add_sync(0xFFFFFFFFu, grew);
+    __shared__ uint32_t part[THREADS / 32];
+    if ((threadIdx.x & 31) == 0) part[threadIdx.x >> 5] = grew;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        uint32_t n = 0;
+        for (int w = 0; w < THREADS / 32; ++w) n += part[w];
+        if (n) atomicAdd(added, n);
+    }
 }
 
 // Level 0: the 1-saddles, if there are any.
-__global__ void reach_start(Summary* sum) { sum->levels = sum->counts[1] > 0 ? 1 : 0; }
+__global__ void reach_start(Summary* sum) {
+    sum->levels = sum->counts[1] > 0 ? 1 : 0;
+    sum->loop_flag[3] = 1;  // the sweeps go on
+}
 
-// End of one loop iteration (two sweeps): the non-empty levels found, and the continue decision
-// (while the second sweep still grew the set, up to the iteration cap).
-__global__ void reach_decide(Summary* sum, int64_t max_iter, cudaGraphConditionalHandle h, int use_handle) {
+// End of one loop iteration (two sweeps): the non-empty levels found, and the continue decision: while
+// the second sweep still added more than `sparse` cells, up to the iteration cap.  The cells it added
+// are what the pushed levels start from.
+__global__ void reach_decide(Summary* sum, uint32_t sparse, int64_t max_iter, cudaGraphConditionalHandle h, int use_handle) {
+    if (!sum->loop_flag[3]) return;
     const uint32_t c0 = sum->loop_flag[0], c1 = sum->loop_flag[1];
     sum->loop_flag[0] = 0;
     sum->loop_flag[1] = 0;
     ++sum->sweep_iters;
     sum->levels += (c0 ? 1 : 0) + (c1 ? 1 : 0);
-    bool more = c1 != 0;
-    if (more && int64_t(sum->levels) >= max_iter) {
+    bool more = c1 > sparse;
+    uint32_t left = more ? 0u : c1;
+    if (c1 && int64_t(sum->levels) >= max_iter) {
         atomicOr(&sum->status, uint32_t(ST_ITER));
         more = false;
+        left = 0;
     }
+    sum->push_count[3] = left;
     sum->loop_flag[3] = more ? 1u : 0u;
     if (use_handle) cudaGraphSetConditional(h, more ? 1u : 0u);
+}
+
+// ---- sparse levels ---------------------------------------------------------------------------
+struct PushArgs {
+    Geom g;
+    const uint32_t* words;
+    uint32_t* reached;     // the bitmap A
+    uint32_t* queue[2];    // handles of a level's new cells
+    uint32_t cap;          // room in each
+    uint32_t* status;
+};
+
+// The targets of cell h's out-edges that were not reached before, marked; returns how many.  The (up to
+// four) atomics go out together, so a level waits for memory once.  LOOK: read the targets' bits
+// first, together too, and mark only those not set -- for large levels, which are bound by the number
+// of atomics and not by one round trip more.
+// The three gradient words that name the targets (the cell's owner and the vertices one step back
+// along the two other axes) are loaded together and the four out-edges computed without branches, for
+// the same reason.
+template <bool LOOK>
+__device__ __forceinline__ int push_cell(const PushArgs& a, uint32_t h, uint32_t out[4]) {
+    const Geom& g = a.g;
+    const uint32_t nx = uint32_t(g.nx), ny = uint32_t(g.ny), nz = uint32_t(g.nz), W = uint32_t(g.W);
+    const uint32_t v = h >> 2;
+    const int axis = int(h & 3u);
+    const uint32_t row = g.div_nx.div(v);
+    const uint32_t x = v - row * nx, z = g.div_ny.div(row), y = row - z * ny;
+    const int bA = axis == 2 ? 0 : axis + 1, bB = axis == 0 ? 2 : axis - 1;
+    const uint32_t cA = pick3(bA, x, y, z), cB = pick3(bB, x, y, z);
+    const uint32_t nA = pick3(bA, nx, ny, nz), nB = pick3(bB, nx, ny, nz);
+    const uint32_t sA = pick3(bA, 1u, nx, nx * ny), sB = pick3(bB, 1u, nx, nx * ny);
+    const uint32_t w_own = __ldg(a.words + v);
+    const uint32_t w_A = cA > 0 ? __ldg(a.words + (v - sA)) : 0u;
+    const uint32_t w_B = cB > 0 ? __ldg(a.words + (v - sB)) : 0u;
+    const uint32_t own = slot_code(w_own, 1 << axis);
+    uint32_t* at[4];
+    uint32_t bit[4], old[4], target[4];
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+        const int b = i < 2 ? bA : bB;
+        const bool plus = i & 1;
+        const uint32_t cb = i < 2 ? cA : cB, nb = i < 2 ? nA : nB;
+        const int other = 3 - axis - b;  // the quad's even axis
+        const uint32_t qc = slot_code(plus ? w_own : (i < 2 ? w_A : w_B), (1 << axis) | (1 << b));
+        const int k = int(qc - 1) >> 1;  // the axis along which the quad is paired
+        const bool edge = (plus ? cb + 1 < nb : cb > 0) && own != uint32_t(1 + 2 * b + (plus ? 1 : 0)) && qc != 0 && k != other;
+        // the facet's owner: the quad's (one step back along b on the - side), one step on along k if
+        // the quad is paired on that side
+        const int back = plus ? 0 : 1, on = (qc & 1u) ? 0 : 1;
+        const uint32_t tx = x - (b == 0 ? back : 0) + (k == 0 ? on : 0), ty = y - (b == 1 ? back : 0) + (k == 1 ? on : 0),
+                       tz = z - (b == 2 ? back : 0) + (k == 2 ? on : 0);
+        const int t_axis = k == axis ? b : axis;
+        target[i] = edge_handle(tx + nx * (ty + ny * tz), t_axis);
+        bit[i] = edge ? 1u << (tx & 31u) : 0u;
+        at[i] = a.reached + (edge ? (((tz * 2 + (t_axis == 2)) * ny + ty) * 2 + (t_axis == 1)) * W + (tx >> 5) : 0u);
+        old[i] = 0;
+    }
+    if (LOOK) {
+#pragma unroll
+        for (int i = 0; i < 4; ++i)
+            if (bit[i]) old[i] = __ldcg(at[i]);
+    }
+#pragma unroll
+    for (int i = 0; i < 4; ++i)
+        if (bit[i] & ~old[i]) old[i] = atomicOr(at[i], bit[i]);
+    int n = 0;
+#pragma unroll
+    for (int i = 0; i < 4; ++i)
+        if (bit[i] & ~old[i]) out[n++] = target[i];
+    return n;
+}
+
+// Exclusive place of n items among the block's (threads in order), and their sum in *total.
+template <int T>
+__device__ __forceinline__ uint32_t block_prefix(uint32_t n, uint32_t* total) {
+    __shared__ uint32_t part[T / 32];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    uint32_t incl = n;
+    for (int o = 1; o < 32; o <<= 1) {
+        const uint32_t y = __shfl_up_sync(0xFFFFFFFFu, incl, o);
+        if (lane >= o) incl += y;
+    }
+    __syncthreads();  // the last call's sums have been read
+    if (lane == 31) part[warp] = incl;
+    __syncthreads();
+    uint32_t w = lane < T / 32 ? part[lane] : 0u;  // every warp scans the warps' sums for itself
+    const uint32_t own = w;
+    for (int o = 1; o < 32; o <<= 1) {
+        const uint32_t y = __shfl_up_sync(0xFFFFFFFFu, w, o);
+        if (lane >= o) w += y;
+    }
+    *total = __shfl_sync(0xFFFFFFFFu, w, T / 32 - 1);
+    return __shfl_sync(0xFFFFFFFFu, w - own, warp) + incl - n;
+}
+
+// The cells of one row word's axis that are set in `bits`, to the queue.
+__device__ __forceinline__ void emit_row(const PushArgs& a, const Rows& r, int axis, uint32_t bits, uint32_t* queue, uint32_t& at) {
+    const uint32_t v0 = vid32(a.g, r.w * 32, r.y, r.z);
+    for (; bits; bits &= bits - 1, ++at)
+        if (at < a.cap) queue[at] = edge_handle(v0 + uint32_t(__ffs(bits) - 1), axis);
+}
+
+// The last swept level's cells (in A but not in B) to queue 0, *count of them (known beforehand).
+__global__ void __launch_bounds__(THREADS) reach_frontier(PushArgs a, const uint32_t* __restrict__ A, const uint32_t* __restrict__ B,
+                                                          const uint32_t* __restrict__ count, uint32_t* __restrict__ cursor) {
+    const uint32_t left = *count;
+    if (!left) return;
+    if (left > a.cap && threadIdx.x == 0) atomicOr(a.status, ST_RETRY);
+    const int64_t nrw = int64_t(a.g.nz) * a.g.ny * a.g.W;
+    __shared__ uint32_t base;
+    for (int64_t t0 = int64_t(blockIdx.x) * THREADS; t0 < nrw; t0 += int64_t(gridDim.x) * THREADS) {
+        const int64_t t = t0 + threadIdx.x;
+        const Rows r(a.g, t < nrw ? t : nrw - 1);
+        uint32_t d[3] = {0, 0, 0};
+        if (t < nrw) {
+            const int e[3] = {r.edge<0>(0, 0), r.edge<1>(0, 0), r.edge<2>(0, 0)};
+#pragma unroll
+            for (int k = 0; k < 3; ++k) d[k] = A[e[k]] & ~B[e[k]];
+        }
+        uint32_t total;
+        uint32_t at = block_prefix<THREADS>(__popc(d[0]) + __popc(d[1]) + __popc(d[2]), &total);
+        if (!total) continue;  // block-uniform
+        if (threadIdx.x == 0) base = atomicAdd(cursor, total);
+        __syncthreads();
+        at += base;
+#pragma unroll
+        for (int k = 0; k < 3; ++k) emit_row(a, r, k, d[k], a.queue[0], at);
+    }
+}
+
+// One pushed level by the whole device: the queue `from` (count push_count[in]) to the other one (count
+// push_count[out]).
+__global__ void __launch_bounds__(THREADS) reach_push(PushArgs a, Summary* sum, int from, int in, int out) {
+    if (pass_retrying(a.status)) return;
+    const uint32_t n = sum->push_count[in];
+    __shared__ uint32_t base;
+    for (uint64_t b = uint64_t(blockIdx.x) * THREADS; b < n; b += uint64_t(gridDim.x) * THREADS) {
+        const uint64_t i = b + threadIdx.x;
+        uint32_t next[4];
+        const int m = i < n ? push_cell<true>(a, a.queue[from][i], next) : 0;
+        uint32_t total;
+        uint32_t at = block_prefix<THREADS>(uint32_t(m), &total);
+        if (threadIdx.x == 0) {
+            base = total ? atomicAdd(&sum->push_count[out], total) : 0u;
+            if (base + total > a.cap) atomicOr(a.status, ST_RETRY);  // the queue is full: the pass sweeps instead
+        }
+        __syncthreads();
+        at += base;
+#pragma unroll
+        for (int k = 0; k < 4; ++k)
+            if (k < m && at + k < a.cap) a.queue[from ^ 1][at + k] = next[k];
+    }
+}
+
+// End of PUSHES pushed levels: those that were not empty, and whether the last one is still too large
+// for one cluster.  An iteration takes push_count[3] in and leaves its levels in 0, 1, 2 and 4.
+constexpr int PUSHES = 4;
+__global__ void reach_push_decide(Summary* sum, uint32_t few, int64_t max_iter, cudaGraphConditionalHandle h, int use_handle) {
+    const uint32_t c[PUSHES] = {sum->push_count[0], sum->push_count[1], sum->push_count[2], sum->push_count[4]};
+    uint32_t left = c[PUSHES - 1];
+    ++sum->push_iters;
+    for (int i = 0; i < PUSHES; ++i) {
+        sum->levels += c[i] ? 1 : 0;
+        if ((i & 1) && c[i] && int64_t(sum->levels) >= max_iter) {  // checked at every second level, as by the sweeps
+            atomicOr(&sum->status, uint32_t(ST_ITER));
+            left = 0;
+            break;
+        }
+    }
+    for (int i = 0; i < 5; ++i) sum->push_count[i] = 0;
+    if (pass_retrying(&sum->status)) left = 0;
+    sum->push_count[3] = left;
+    const bool more = left > few;
+    sum->loop_flag[3] = more ? 1u : 0u;
+    if (use_handle) cudaGraphSetConditional(h, more ? 1u : 0u);
+}
+
+// The remaining levels in one cluster of thread blocks: queue 0 holds the current level, or (`all`)
+// the levels start here, from every cell of the bitmap (the 1-saddles).  The counts live in the first
+// block's shared memory; a cluster barrier ends each level.
+constexpr int TAIL_THREADS = 1024;
+__global__ void __launch_bounds__(TAIL_THREADS, 1) reach_tail(PushArgs a, Summary* sum, int all, int64_t max_iter) {
+    cg::cluster_group cluster = cg::this_cluster();
+    __shared__ uint32_t counts[3], state[2], alone[TAIL_THREADS];
+    __shared__ uint64_t state_levels, block_levels;
+    __shared__ uint32_t base, level_n;
+    uint32_t* const shared_counts = cluster.map_shared_rank(counts, 0);
+    const uint32_t rank = cluster.block_rank(), size = cluster.num_blocks();
+    if (threadIdx.x < 3) counts[threadIdx.x] = 0;
+    cluster.sync();
+    uint32_t n = sum->push_count[3];
+    if (all) {
+        const int64_t nrw = int64_t(a.g.nz) * a.g.ny * a.g.W;
+        for (int64_t t0 = int64_t(rank) * TAIL_THREADS; t0 < nrw; t0 += int64_t(size) * TAIL_THREADS) {
+            const int64_t t = t0 + threadIdx.x;
+            const Rows r(a.g, t < nrw ? t : nrw - 1);
+            uint32_t d[3] = {0, 0, 0};
+            if (t < nrw) {
+                d[0] = a.reached[r.edge<0>(0, 0)];
+                d[1] = a.reached[r.edge<1>(0, 0)];
+                d[2] = a.reached[r.edge<2>(0, 0)];
+            }
+            uint32_t total;
+            uint32_t at = block_prefix<TAIL_THREADS>(__popc(d[0]) + __popc(d[1]) + __popc(d[2]), &total);
+            if (!total) continue;  // block-uniform
+            if (threadIdx.x == 0) base = atomicAdd(&shared_counts[2], total);
+            __syncthreads();
+            at += base;
+#pragma unroll
+            for (int k = 0; k < 3; ++k) emit_row(a, r, k, d[k], a.queue[0], at);
+        }
+        cluster.sync();
+        if (threadIdx.x == 0) level_n = shared_counts[2];
+        __syncthreads();
+        n = level_n;
+    }
+    // level k reads queue k & 1 and counts its new cells in counts[k % 3]; counts[(k + 1) % 3], last read
+    // before level k - 1 began, is cleared for the next level
+    uint64_t levels = sum->levels;
+    cluster.sync();  // every block has read the counts and the level number
+    for (int k = 0; n;) {
+        n = min(n, a.cap);
+        if (n <= TAIL_THREADS) {
+            // the first block goes on alone, with the level in its shared memory and no barrier but its
+            // own, until the levels end or one outgrows its threads (that one goes to the queue); the others
+            // wait at the cluster's barrier
+            if (rank == 0) {
+                uint32_t h = threadIdx.x < n ? a.queue[k & 1][threadIdx.x] : 0u;
+                for (;;) {
+                    uint32_t next[4], total;
+                    const int m = threadIdx.x < n ? push_cell<false>(a, h, next) : 0;
+                    const uint32_t at = block_prefix<TAIL_THREADS>(uint32_t(m), &total);
+                    ++k;
+                    n = total;
+                    levels += n ? 1 : 0;
+                    if (!(k & 1) && n && int64_t(levels) >= max_iter) {  // at every second level, as the sweeps
+                        if (threadIdx.x == 0) atomicOr(a.status, ST_ITER);
+                        n = 0;
+                    }
+                    if (!n) break;
+                    uint32_t* to = n > TAIL_THREADS ? a.queue[k & 1] : alone;
+                    if (n > a.cap && threadIdx.x == 0) atomicOr(a.status, ST_RETRY);
+#pragma unroll
+                    for (int j = 0; j < 4; ++j)
+                        if (j < m && at + j < a.cap) to[at + j] = next[j];
+                    if (n > TAIL_THREADS) break;
+                    __syncthreads();
+                    h = threadIdx.x < n ? alone[threadIdx.x] : 0u;
+                }
+                if (threadIdx.x == 0) {
+                    state[0] = n;
+                    state[1] = uint32_t(k);
+                    state_levels = levels;
+                    counts[0] = counts[1] = counts[2] = 0;
+                }
+            }
+            cluster.sync();
+            if (threadIdx.x == 0) {
+                level_n = *cluster.map_shared_rank(&state[0], 0);
+                base = *cluster.map_shared_rank(&state[1], 0);
+                block_levels = *cluster.map_shared_rank(&state_levels, 0);
+            }
+            __syncthreads();
+            n = level_n;
+            k = int(base);
+            levels = block_levels;
+            cluster.sync();  // the first block may change its state again
+            continue;
+        }
+        if (rank == 0 && threadIdx.x == 0) counts[(k + 1) % 3] = 0;
+        const uint32_t* from = a.queue[k & 1];
+        uint32_t* to = a.queue[(k & 1) ^ 1];
+        for (uint32_t b = rank * TAIL_THREADS; b < n; b += size * TAIL_THREADS) {
+            uint32_t next[4];
+            const int m = b + threadIdx.x < n ? push_cell<false>(a, from[b + threadIdx.x], next) : 0;
+            uint32_t total;
+            uint32_t at = block_prefix<TAIL_THREADS>(uint32_t(m), &total);
+            if (!total) continue;  // block-uniform
+            if (threadIdx.x == 0) {
+                base = atomicAdd(&shared_counts[k % 3], total);
+                if (base + total > a.cap) atomicOr(a.status, ST_RETRY);
+            }
+            __syncthreads();
+            at += base;
+#pragma unroll
+            for (int j = 0; j < 4; ++j)
+                if (j < m && at + j < a.cap) to[at + j] = next[j];
+        }
+        cluster.sync();
+        if (threadIdx.x == 0) level_n = shared_counts[k % 3];
+        __syncthreads();
+        n = level_n;
+        ++k;
+        levels += n ? 1 : 0;
+        if (!(k & 1) && n && int64_t(levels) >= max_iter) {
+            if (rank == 0 && threadIdx.x == 0) atomicOr(a.status, ST_ITER);
+            n = 0;
+        }
+    }
+    if (rank == 0 && threadIdx.x == 0) sum->levels = levels;
+    cluster.sync();  // no block leaves while others read the first one's counts
 }
 
 // Down-quad bits of the quads with even axis K owned by vertex (x + DX, y + DY, z + DZ).
@@ -387,19 +716,83 @@ int grid_for(const Plan* p, int64_t threads) {
     return int(std::max<int64_t>(1, std::min(want, cap)));
 }
 
+// Grids of at most this many row words push every level in one cluster: 0.072 ms against 0.127 by
+// sweeps on a 1024-word lattice, but 0.164 against 0.072 (two sweep iterations, then the cluster) on a
+// 7350-word GRF, whose first levels have 100 thousand cells.
+constexpr int64_t TAIL_ROW_WORDS = 2048;
+// A level of at most this many new cells is left to one cluster (two cells a thread; 128 thousand, eight
+// a thread, took 1.5 ms of the 512^3 blob field's levels that the whole device pushes in 0.6 ms) ...
+constexpr uint32_t TAIL_CELLS = 32 * 1024;
+// ... and one of at most a third of a cell per row word is pushed rather than swept: a sweep takes some
+// 25 ps a row word, a pushed level some 60 ps a cell and its launch.
+constexpr int64_t SPARSE_DIV = 3;
+
 struct SweepCtx {
     dim3 grid;
     const uint4* masks;
     uint32_t* a;
     uint32_t* b;
     uint32_t* stamp;
+    uint32_t sparse;
 };
 
 void sweep_body(Plan* p, cudaStream_t s, cudaGraphConditionalHandle h, void* ctx) {
     const SweepCtx& c = *static_cast<SweepCtx*>(ctx);
     reach_sweep<<<c.grid, THREADS, 0, s>>>(p->g, c.masks, c.a, c.b, c.stamp, p->dsum(), 0, &p->dsum()->loop_flag[0]);
     reach_sweep<<<c.grid, THREADS, 0, s>>>(p->g, c.masks, c.b, c.a, c.stamp, p->dsum(), 1, &p->dsum()->loop_flag[1]);
-    reach_decide<<<1, 1, 0, s>>>(p->dsum(), p->opts.max_iterations, h, h != 0);
+    reach_decide<<<1, 1, 0, s>>>(p->dsum(), c.sparse, p->opts.max_iterations, h, h != 0);
+}
+
+struct PushCtx {
+    int grid;
+    PushArgs a;
+};
+
+void push_body(Plan* p, cudaStream_t s, cudaGraphConditionalHandle h, void* ctx) {
+    const PushCtx& c = *static_cast<PushCtx*>(ctx);
+    for (int i = 0; i < PUSHES; ++i)
+        reach_push<<<c.grid, THREADS, 0, s>>>(c.a, p->dsum(), i & 1, i == 0 ? 3 : i - 1, i == PUSHES - 1 ? 4 : i);
+    reach_push_decide<<<1, 1, 0, s>>>(p->dsum(), TAIL_CELLS, p->opts.max_iterations, h, h != 0);
+}
+
+// One cluster over as many blocks as this device can schedule together.
+msc_status launch_tail(Plan* p, cudaStream_t s, const PushArgs& a, int all) {
+    msc_status st;
+    if (!p->tail_cluster) {
+        if ((st = check_cuda(p, cudaFuncSetAttribute(reach_tail, cudaFuncAttributeNonPortableClusterSizeAllowed, 1),
+                             "cudaFuncSetAttribute(reach_tail)")))
+            return st;
+        for (int size : {16, 8, 4, 2, 1}) {
+            cudaLaunchConfig_t cfg{};
+            cfg.gridDim = dim3(unsigned(size));
+            cfg.blockDim = dim3(TAIL_THREADS);
+            cudaLaunchAttribute at{};
+            at.id = cudaLaunchAttributeClusterDimension;
+            at.val.clusterDim.x = unsigned(size);
+            at.val.clusterDim.y = at.val.clusterDim.z = 1;
+            cfg.attrs = &at;
+            cfg.numAttrs = 1;
+            int n = 0;
+            if (cudaOccupancyMaxActiveClusters(&n, reach_tail, &cfg) == cudaSuccess && n > 0) {
+                p->tail_cluster = size;
+                break;
+            }
+            cudaGetLastError();
+        }
+        if (!p->tail_cluster) return fail(p, MSC_ERR_CUDA, "no thread-block cluster can be launched");
+    }
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = dim3(unsigned(p->tail_cluster));
+    cfg.blockDim = dim3(TAIL_THREADS);
+    cfg.stream = s;
+    cudaLaunchAttribute at{};
+    at.id = cudaLaunchAttributeClusterDimension;
+    at.val.clusterDim.x = unsigned(p->tail_cluster);
+    at.val.clusterDim.y = at.val.clusterDim.z = 1;
+    cfg.attrs = &at;
+    cfg.numAttrs = 1;
+    launched(p);
+    return check_cuda(p, cudaLaunchKernelEx(&cfg, reach_tail, a, p->dsum(), all, p->opts.max_iterations), "reach_tail launch");
 }
 
 }  // namespace
@@ -431,8 +824,60 @@ msc_status run_reachability(Plan* p, cudaStream_t s) {
     // longer CTAs would cost little alone but leave long tails when other passes share the device.
     const int64_t tiles = (nrw + THREADS - 1) / THREADS;
     const int64_t sweep_ctas = std::min<int64_t>(tiles, std::max<int64_t>(int64_t(std::max(1, p->num_sms)) * 4, (tiles + 3) / 4));
-    SweepCtx ctx{dim3(unsigned(std::max<int64_t>(1, sweep_ctas)), 1), masks, A, B, stamp};
-    return run_loop(p, s, 1, 3, sweep_body, &ctx);
+    SweepCtx ctx{dim3(unsigned(std::max<int64_t>(1, sweep_ctas)), 1), masks, A, B, stamp, 0};
+    if (p->reach_sweeps_only) return run_loop(p, s, 1, 3, sweep_body, &ctx);
+    // the pushed levels.  A small grid's queues hold every 1-cell; a large one's twelve times the level
+    // they start from (a level of a sparse front hardly grows), and a pass that needs more asks for a
+    // rerun by sweeps alone
+    const bool all = nrw <= TAIL_ROW_WORDS;
+    const int64_t sparse = std::max<int64_t>(TAIL_CELLS, nrw / SPARSE_DIV);
+    const int64_t room = all ? 3 * g.nverts : 12 * sparse;
+    if ((st = ensure(p, p->reach_queue, sizeof(uint32_t) * 2 * size_t(room)))) return st;
+    PushArgs a{};
+    a.g = g;
+    a.words = static_cast<const uint32_t*>(p->words.ptr);
+    a.reached = A;
+    a.queue[0] = static_cast<uint32_t*>(p->reach_queue.ptr);
+    a.queue[1] = a.queue[0] + room;
+    a.cap = uint32_t(room);
+    a.status = p->status_word();
+    if (!all) {
+        ctx.sparse = uint32_t(sparse);
+        if (!p->capturing) {
+            if ((st = run_loop(p, s, 1, 3, sweep_body, &ctx))) return st;
+        } else {
+            // as many iterations as the last synchronised pass took, one after another (a conditional
+            // node costs 12 us an iteration): a field that needs fewer skips the rest, one that needs
+            // more pushes a larger level
+            for (int64_t i = 0; i < p->reach_iters; ++i) {
+                if (i + 1 == p->reach_iters) ctx.sparse = 0xFFFFFFFFu;
+                sweep_body(p, s, 0, &ctx);
+                launched(p, 3);
+            }
+            p->loop_body_launches[1] = 0;
+        }
+        Summary* sum = p->dsum();
+        reach_frontier<<<grid_for(p, nrw), THREADS, 0, s>>>(a, A, B, &sum->push_count[3], &sum->push_cursor);
+        launched(p);
+        if (sparse > TAIL_CELLS) {
+            PushCtx pc{std::max(1, p->num_sms) * 8, a};
+            if ((st = run_loop(p, s, 3, PUSHES + 1, push_body, &pc))) return st;
+        }
+    }
+    if ((st = launch_tail(p, s, a, all ? 1 : 0))) return st;
+    if (p->capturing) return MSC_OK;
+    // a synchronised pass whose queue was full (a replayed one comes here through its rerun)
+    if ((st = read_summary(p, s))) return st;
+    p->reach_iters = std::max<int64_t>(1, int64_t(p->hsum->sweep_iters));
+    if (!(p->hsum->status & ST_RETRY)) return MSC_OK;
+    p->reach_sweeps_only = true;
+    const uint32_t clear[2] = {p->hsum->status & ~uint32_t(ST_RETRY), 0u};
+    if ((st = check_cuda(p, cudaMemcpyAsync(p->status_word(), &clear[0], sizeof(uint32_t), cudaMemcpyHostToDevice, s), "status reset")) ||
+        (st = check_cuda(p, cudaMemsetAsync(&p->dsum()->sweep_iters, 0, sizeof(unsigned long long), s), "loop reset")) ||
+        (st = check_cuda(p, cudaMemsetAsync(p->dsum()->push_count, 0, sizeof(p->dsum()->push_count), s), "loop reset")) ||
+        (st = check_cuda(p, cudaStreamSynchronize(s), "stream sync")))
+        return st;
+    return run_reachability(p, s);
 }
 
 msc_status run_junctions(Plan* p, cudaStream_t s) {

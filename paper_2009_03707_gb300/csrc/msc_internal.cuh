@@ -42,6 +42,7 @@ __device__ __forceinline__ bool count_fits(uint32_t* status, unsigned long long 
 // Path-count counter slots in Summary::pc.
 enum PcCounter { PC_CURSOR = 0, PC_MAX = 1, PC_ITER = 2, PC_ENTRIES = 3, PC_DEFER0 = 4, PC_DEFER1 = 5, PC_NEXT = 6,
                  PC_DEFER2 = 7, PC_DEFER3 = 8, PC_NEXT_GROUP = 9, PC_NEXT_WARP = 10, PC_SLOTS = 12 };
+constexpr int DP_WAVES = 8;  // waves of the junction DP per iteration of its loop (even)
 struct Summary {
     unsigned long long counts[4];     // critical cells per dimension
     unsigned long long n_junctions;
@@ -52,13 +53,11 @@ struct Summary {
     unsigned long long minor_nnz[4];  // distinct entries of A, B, B*, D
     unsigned long long pc[PC_SLOTS];  // path-count counters (PcCounter)
     unsigned long long dstar_nnz;
-    unsigned long long dp_wave_done;      // junction DP: junctions done in the current wave
     unsigned long long dp_pool_used;      // junction DP: J-row pool slots taken
     unsigned long long dp_junctions_done;
     unsigned long long dp_iters;          // iterations of the wave loop
-    unsigned long long dp_long_n;         // junction DP: long merges handed to the warp kernel this wave
-    unsigned int dp_wave;                 // the current wave
-    unsigned int pad2;
+    uint32_t dp_queue[DP_WAVES + 1];      // junction DP: junctions of the loop iteration's waves and the next one's
+    uint32_t pad2;
     uint32_t loop_flag[4];            // "changed" flags of the iterative stages; [3] = continue (host loops)
     uint32_t status;                  // StatusBit word
     uint32_t pad;
@@ -104,7 +103,7 @@ struct Plan {
     // counts the host reads
     DeviceBuffer simp_alive, simp_node, simp_len, simp_pos, simp_scan;
     DeviceBuffer simp_ptr, simp_nbr[2], simp_mult[2], simp_log, simp_sort, simp_round;
-    DeviceBuffer dp_pend, dp_in_cnt, dp_in_ptr, dp_in_idx, dp_j_off, dp_j_len, dp_pool_col, dp_pool_cnt, dp_long, dp_chunks;
+    DeviceBuffer dp_pend, dp_in_cnt, dp_in_ptr, dp_in_idx, dp_j_off, dp_j_len, dp_pool_col, dp_pool_cnt, dp_queues;
 
     template <class F>
     void for_each_buffer(F&& f) {
@@ -116,7 +115,7 @@ struct Plan {
                                &minor_mult[0], &minor_mult[1], &minor_mult[2], &minor_mult[3], &pc_rowstart, &pc_rowlen,
                                &pc_big, &pc_col, &pc_cnt, &pc_gk, &pc_gv, &pc_gocc, &dstar_rowptr, &dstar_col,
                                &dstar_count, &dp_pend, &dp_in_cnt, &dp_in_ptr, &dp_in_idx, &dp_j_off,
-                               &dp_j_len, &dp_pool_col, &dp_pool_cnt, &dp_long, &dp_chunks, &csc_colptr, &csc_row, &csc_count, &csc_work,
+                               &dp_j_len, &dp_pool_col, &dp_pool_cnt, &dp_queues, &csc_colptr, &csc_row, &csc_count, &csc_work,
                                &graph_nodeptr, &graph_adj, &graph_mult, &graph_work, &graph_none,
                                &geo_len, &geo_off, &geo_scan, &geo_cells, &ss_len, &ss_off, &ss_scan, &ss_cells, &ss_row,
                                &simp_alive, &simp_node, &simp_len, &simp_pos, &simp_scan,

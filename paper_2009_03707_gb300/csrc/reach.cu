@@ -668,7 +668,7 @@ __device__ __forceinline__ void classify_axis(const Geom& g, const Rows& r, int 
     }
     if (x < g.nx) info[info_index(g, edge_handle(v, A))] = rec;
     const uint32_t jw = __ballot_sync(0xFFFFFFFFu, mine && n > 1);
-    if (lane == 0) junc[r.edge<A>(0, 0)] = jw;
+    if (lane == 0) junc[A * r.qplane + r.qbase] = jw;
 }
 
 // One warp per vertex-row word, all three axes: every load of the word (the bitmaps of the three
@@ -698,7 +698,6 @@ __global__ void __launch_bounds__(THREADS, 4) classify_reached(Geom g, const uin
         classify_axis<0>(g, r, lane, x, v, i0, w0, wy, wz, info, junc, cnt);
         classify_axis<1>(g, r, lane, x, v, i1, w0, wx, wz, info, junc, cnt);
         classify_axis<2>(g, r, lane, x, v, i2, w0, wx, wy, info, junc, cnt);
-        if (lane == 0) junc[g.edge_word(r.z, 1, r.y, 1, r.w)] = 0;  // the unused slot of the 1-cell layout
     }
     __shared__ unsigned long long part[THREADS / 32];
     if (lane == 0) part[threadIdx.x >> 5] = cnt;
@@ -883,11 +882,10 @@ msc_status run_reachability(Plan* p, cudaStream_t s) {
 msc_status run_junctions(Plan* p, cudaStream_t s) {
     const Geom& g = p->g;
     msc_status st;
-    const int64_t nw = g.edge_words();
-    if ((st = ensure(p, p->junc_bits, sizeof(uint32_t) * size_t(nw)))) return st;
-    if ((st = ensure(p, p->junc_prefix, sizeof(uint32_t) * size_t(nw)))) return st;
-    if ((st = ensure(p, p->node_info, sizeof(uint32_t) * 3 * size_t(g.nverts)))) return st;
     const int64_t nrw = int64_t(g.nz) * g.ny * g.W;
+    if ((st = ensure(p, p->junc_bits, sizeof(uint32_t) * 3 * size_t(nrw)))) return st;
+    if ((st = ensure(p, p->junc_prefix, sizeof(uint32_t) * 3 * size_t(nrw)))) return st;
+    if ((st = ensure(p, p->node_info, sizeof(uint32_t) * 3 * size_t(g.nverts)))) return st;
     classify_reached<<<grid_for(p, nrw * 32), THREADS, 0, s>>>(
         g, static_cast<const uint32_t*>(p->words.ptr), static_cast<const uint32_t*>(p->visited.ptr),
         static_cast<const uint4*>(p->reach_masks.ptr), static_cast<const uint32_t*>(p->reach_qdown.ptr),

@@ -71,8 +71,8 @@ struct CritSource {
     }
 };
 
-// 1-cells marked in a bitmap stored directly in the 1-cell row layout (a = 1-b-c): one
-// sequence, word index = i, ids to out.
+// 1-cells marked in one bitmap per axis, [axis][z][y][w] (the critical bitmaps' layout, so that a
+// 1-cell's word follows from its owner's row): one sequence, ids to out.
 struct EdgeSource {
     Geom g;
     const uint32_t* bits;
@@ -82,7 +82,7 @@ struct EdgeSource {
     uint32_t* status;
     __device__ int64_t word_index(int, int64_t i) const {
         RowCoord r = decode_row(g, i);
-        return (r.b & r.c) ? -1 : i;
+        return (r.b & r.c) ? -1 : g.slot_word(r.b + 2 * r.c, r.z, r.y, r.w);
     }
     __device__ void emit(int, int64_t i, uint64_t pos, uint32_t word) const {
         RowCoord r = decode_row(g, i);

@@ -268,9 +268,8 @@ msc_status run_critical(Plan* p, cudaStream_t s) {
 // atomically.
 msc_status enqueue_pipeline(Plan* p, const float* d_field, cudaStream_t s, bool branch) {
     msc_status st;
-    if ((st = check_cuda(p, cudaMemsetAsync(p->dsum(), 0, sizeof(Summary), s), "summary clear"))) return st;
     stage_start(p, 0, s);
-    if ((st = run_gradient(p, d_field, s))) return st;
+    if ((st = run_gradient(p, d_field, s))) return st;  // its first kernel clears the summary
     stage_end(p, 0, s);
     stage_start(p, 1, s);
     if ((st = run_critical(p, s))) return st;
@@ -296,7 +295,13 @@ msc_status enqueue_pipeline(Plan* p, const float* d_field, cudaStream_t s, bool 
     stage_start(p, 5, s);
     if ((st = run_path_count(p, s))) return st;
     stage_end(p, 5, s);
-    return branch ? check_cuda(p, cudaStreamWaitEvent(s, p->join_ev, 0), "join") : MSC_OK;
+    if (branch && (st = check_cuda(p, cudaStreamWaitEvent(s, p->join_ev, 0), "join"))) return st;
+    if (!p->capturing) return MSC_OK;
+    for (int k = 0; k <= int(branch); ++k)  // the timing branches end with the pass
+        if ((st = check_cuda(p, cudaEventRecord(p->timing_ev, p->timing_stream[k]), "join")) ||
+            (st = check_cuda(p, cudaStreamWaitEvent(s, p->timing_ev, 0), "join")))
+            return st;
+    return MSC_OK;
 }
 
 void destroy_graph(Plan* p) {
@@ -429,6 +434,9 @@ msc_status msc_plan(const int64_t dims[3], const msc_opts* opts, msc_plan_t* out
     if (!st) st = msc::check_cuda(p, cudaStreamCreateWithPriority(&p->body_stream, cudaStreamNonBlocking, hi_prio), "cudaStreamCreate");
     if (!st) st = msc::check_cuda(p, cudaStreamCreateWithPriority(&p->side_stream, cudaStreamNonBlocking, lo_prio), "cudaStreamCreate");
     if (!st) st = msc::check_cuda(p, cudaStreamCreateWithPriority(&p->side_body_stream, cudaStreamNonBlocking, lo_prio), "cudaStreamCreate");
+    for (cudaStream_t& t : p->timing_stream)
+        if (!st) st = msc::check_cuda(p, cudaStreamCreateWithPriority(&t, cudaStreamNonBlocking, lo_prio), "cudaStreamCreate");
+    if (!st) st = msc::check_cuda(p, cudaEventCreateWithFlags(&p->timing_ev, cudaEventDisableTiming), "cudaEventCreate");
     if (!st) st = msc::check_cuda(p, cudaEventCreateWithFlags(&p->fork_ev, cudaEventDisableTiming), "cudaEventCreate");
     if (!st) st = msc::check_cuda(p, cudaEventCreateWithFlags(&p->join_ev, cudaEventDisableTiming), "cudaEventCreate");
     if (!st) st = msc::check_cuda(p, cudaMallocHost(&p->hsum, sizeof(msc::Summary)), "cudaMallocHost");
@@ -454,9 +462,9 @@ msc_status msc_plan_destroy(msc_plan_t plan) {
     });
     for (cudaEvent_t e : p->stage_ev)
         if (e) cudaEventDestroy(e);
-    for (cudaEvent_t e : {p->kev0, p->kev1, p->tev0, p->tev1, p->gev0, p->gev1, p->pend_ev, p->fork_ev, p->join_ev})
+    for (cudaEvent_t e : {p->kev0, p->kev1, p->tev0, p->tev1, p->gev0, p->gev1, p->pend_ev, p->fork_ev, p->join_ev, p->timing_ev})
         if (e) cudaEventDestroy(e);
-    for (cudaStream_t t : {p->cap_stream, p->body_stream, p->side_stream, p->side_body_stream})
+    for (cudaStream_t t : {p->cap_stream, p->body_stream, p->side_stream, p->side_body_stream, p->timing_stream[0], p->timing_stream[1]})
         if (t) cudaStreamDestroy(t);
     if (p->hsum) cudaFreeHost(p->hsum);
     delete p;

@@ -280,8 +280,12 @@ __global__ void __launch_bounds__(256) critical_bitmaps(Geom g, const uint32_t* 
 // Zeroes the words that the lower-star kernel finishes with atomicOr: those on the + faces of its
 // tiles (x = 31 mod 32, y = TY-1 mod TY, z = TZ-1 mod TZ), which receive codes from the next tiles'
 // stars.  Every other word gets one plain store, so it needs no zeroing.  A warp per (y, z) row:
-// a row on a y or z face is cleared whole, any other row only at x = 31 mod 32.
-__global__ void __launch_bounds__(256) zero_face_words(Geom g, uint32_t* __restrict__ words, int ty, int tz) {
+// a row on a y or z face is cleared whole, any other row only at x = 31 mod 32.  As the first kernel of a
+// replayed pass it also clears the pass's summary (a memset node before it cost 8 us).
+__global__ void __launch_bounds__(256) zero_face_words(Geom g, uint32_t* __restrict__ words, int ty, int tz,
+                                                       uint32_t* __restrict__ summary) {
+    if (summary && blockIdx.x == 0)
+        for (uint32_t i = threadIdx.x; i < uint32_t(sizeof(Summary) / sizeof(uint32_t)); i += blockDim.x) summary[i] = 0;
     const uint32_t row = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;  // ny * nz < 2^31
     const int lane = threadIdx.x & 31;
     if (row >= uint32_t(g.ny) * uint32_t(g.nz)) return;  // warp-uniform
@@ -314,10 +318,11 @@ cudaError_t launch_tile(const Geom& g, const float* d_field, uint32_t* words, ui
     return cudaGetLastError();
 }
 
-cudaError_t launch_zero_faces(int v, const Geom& g, uint32_t* words, cudaStream_t s) {
+cudaError_t launch_zero_faces(int v, const Geom& g, uint32_t* words, cudaStream_t s, Summary* clear = nullptr) {
     if (v < 0 || v >= N_VARIANTS) v = 0;
     const int64_t rows = int64_t(g.ny) * g.nz;
-    zero_face_words<<<unsigned((rows * 32 + 255) / 256), 256, 0, s>>>(g, words, VARIANTS[v].ty, VARIANTS[v].tz);
+    zero_face_words<<<unsigned((rows * 32 + 255) / 256), 256, 0, s>>>(g, words, VARIANTS[v].ty, VARIANTS[v].tz,
+                                                                        reinterpret_cast<uint32_t*>(clear));
     return cudaGetLastError();
 }
 
@@ -341,7 +346,7 @@ cudaError_t launch_words(int v, const Geom& g, const float* d_field, uint32_t* w
 
 cudaError_t launch_gradient(int v, const Geom& g, const float* d_field, uint32_t* words, uint32_t* crit_bits,
                             uint32_t* status, cudaStream_t s, const Plan* p = nullptr) {
-    cudaError_t e = launch_zero_faces(v, g, words, s);
+    cudaError_t e = launch_zero_faces(v, g, words, s, p && p->capturing ? p->dsum() : nullptr);
     if (e != cudaSuccess) return e;
     if (p) record_event(p, p->gev0, s);  // the lower-star kernel alone is timed
     switch (v) {

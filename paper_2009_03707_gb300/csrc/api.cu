@@ -711,7 +711,7 @@ msc_status msc_arc_geometry(msc_plan_t plan, msc_stream_t stream, int64_t* n_arc
 }
 
 // The cells of the saddle-saddle arcs of multiplicity 1 need the rows of J.  A pass that counted
-// paths row by row has none, so the junction waves run once more for them (they give the same D*);
+// paths row by row has none, so the junction waves run once more for them, without the D* rows;
 // the pass's summary, statistics and kernel timings are put back afterwards.
 static msc_status ensure_ss_geometry(Plan* p, cudaStream_t s) {
     msc_status st;
@@ -726,7 +726,9 @@ static msc_status ensure_ss_geometry(Plan* p, cudaStream_t s) {
         cudaEvent_t k0 = p->kev0, k1 = p->kev1;
         p->kev0 = p->kev1 = nullptr;
         p->opts.path_count_method = 2;
+        p->j_only = true;
         st = msc::run_path_count(p, s);
+        p->j_only = false;
         if (st == MSC_OK) st = msc::finish_stage(p, s);
         p->opts.path_count_method = forced;
         p->pc_method_used = used;

@@ -550,7 +550,8 @@ void wave_body(Plan* p, cudaStream_t s, cudaGraphConditionalHandle h, void* ctx)
 
 }  // namespace
 
-// Enqueues the junction DP and the D* rows into staging (the caller scans and gathers them).
+// Enqueues the junction DP and, unless only J is wanted, the D* rows into staging (the caller scans and
+// gathers them).
 // pool_cap / out_cap: capacities of the J-row pool and of the staging.
 msc_status run_junction_dp(Plan* p, cudaStream_t s, uint64_t pool_cap, uint64_t out_cap) {
     msc_status st;
@@ -566,7 +567,9 @@ msc_status run_junction_dp(Plan* p, cudaStream_t s, uint64_t pool_cap, uint64_t 
     if ((st = ensure(p, p->dp_j_len, sizeof(uint32_t) * njc))) return st;
     if ((st = ensure(p, p->dp_pool_col, sizeof(uint32_t) * size_t(pool_cap ? pool_cap : 1)))) return st;
     if ((st = ensure(p, p->dp_pool_cnt, sizeof(u64) * size_t(pool_cap ? pool_cap : 1)))) return st;
-    if ((st = ensure(p, p->minor_scan, std::max(row_scan_scratch_bytes(capj), row_scan_scratch_bytes(cap1))))) return st;
+    // a scratch of its own: a captured pass keeps pointers to minor_scan, which must not grow for a J asked
+    // for between its replays
+    if ((st = ensure(p, p->dp_scan, row_scan_scratch_bytes(capj)))) return st;
     DpArgs a{};
     a.tgt = static_cast<const uint32_t*>(p->trace.ptr);
     a.kinds = static_cast<const uint32_t*>(p->trace_kinds.ptr);
@@ -602,7 +605,7 @@ msc_status run_junction_dp(Plan* p, cudaStream_t s, uint64_t pool_cap, uint64_t 
     const int gj = grid_cap(p, capj, THREADS, 8);
     dp_init<<<gj, THREADS, 0, s>>>(a);
     launched(p);
-    if ((st = check_cuda(p, row_scan(p, a.in_cnt, a.nj_dev, capj, a.in_ptr, static_cast<u64*>(p->minor_scan.ptr), s),
+    if ((st = check_cuda(p, row_scan(p, a.in_cnt, a.nj_dev, capj, a.in_ptr, static_cast<u64*>(p->dp_scan.ptr), s),
                          "predecessor scan")))
         return st;
     dp_fill<<<gj, THREADS, 0, s>>>(a);
@@ -611,6 +614,7 @@ msc_status run_junction_dp(Plan* p, cudaStream_t s, uint64_t pool_cap, uint64_t 
     record_event(p, p->kev0, s);
     WaveCtx ctx{grid_cap(p, capj, 4, 8), a};
     if ((st = run_loop(p, s, 2, WAVES + 1, wave_body, &ctx))) return st;
+    if (p->j_only) return MSC_OK;
     dp_rows<<<grid_cap(p, cap1, THREADS, 8), THREADS, 0, s>>>(a);
     record_event(p, p->kev1, s);
     launched(p);

@@ -103,7 +103,7 @@ struct Plan {
     // counts the host reads
     DeviceBuffer simp_alive, simp_node, simp_len, simp_pos, simp_scan;
     DeviceBuffer simp_ptr, simp_nbr[2], simp_mult[2], simp_log, simp_sort, simp_round;
-    DeviceBuffer dp_pend, dp_in_cnt, dp_in_ptr, dp_in_idx, dp_j_off, dp_j_len, dp_pool_col, dp_pool_cnt, dp_queues;
+    DeviceBuffer dp_pend, dp_in_cnt, dp_in_ptr, dp_in_idx, dp_j_off, dp_j_len, dp_pool_col, dp_pool_cnt, dp_queues, dp_scan;
 
     template <class F>
     void for_each_buffer(F&& f) {
@@ -115,7 +115,7 @@ struct Plan {
                                &minor_mult[0], &minor_mult[1], &minor_mult[2], &minor_mult[3], &pc_rowstart, &pc_rowlen,
                                &pc_big, &pc_col, &pc_cnt, &pc_gk, &pc_gv, &pc_gocc, &dstar_rowptr, &dstar_col,
                                &dstar_count, &dp_pend, &dp_in_cnt, &dp_in_ptr, &dp_in_idx, &dp_j_off,
-                               &dp_j_len, &dp_pool_col, &dp_pool_cnt, &dp_queues, &csc_colptr, &csc_row, &csc_count, &csc_work,
+                               &dp_j_len, &dp_pool_col, &dp_pool_cnt, &dp_queues, &dp_scan, &csc_colptr, &csc_row, &csc_count, &csc_work,
                                &graph_nodeptr, &graph_adj, &graph_mult, &graph_work, &graph_none,
                                &geo_len, &geo_off, &geo_scan, &geo_cells, &ss_len, &ss_off, &ss_scan, &ss_cells, &ss_row,
                                &simp_alive, &simp_node, &simp_len, &simp_pos, &simp_scan,
@@ -167,6 +167,7 @@ struct Plan {
     int64_t dp_pool_cap = 0;     // J-row pool slots of the last junction-DP run
     int pc_method_chosen = 0;    // path-count method once the first run has measured the minor (1, 2)
     int pc_method_used = 0;      // the method of the last run
+    bool j_only = false;         // the run in hand is for the rows of J; the pass's D* stays as it is
     // which stages are valid for the current field
     bool have_gradient = false, have_critical = false, have_extremum = false, have_reach = false,
          have_junctions = false, have_trace = false, have_minor = false, have_dstar = false,

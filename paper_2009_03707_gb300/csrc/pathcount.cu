@@ -933,10 +933,10 @@ msc_status run_path_count(Plan* p, cudaStream_t s) {
         uint64_t pool = cap_mode ? uint64_t(p->caps.dp_pool)
                                  : uint64_t(std::max<int64_t>(p->dp_pool_cap, 4 * njcap + 1024));
         for (int attempt = 0; attempt < 8; ++attempt) {
-            if ((st = ensure(p, p->pc_col, sizeof(uint32_t) * cap))) return st;
-            if ((st = ensure(p, p->pc_cnt, sizeof(u64) * cap))) return st;
-            if ((st = ensure(p, p->dstar_col, sizeof(uint32_t) * cap))) return st;
-            if ((st = ensure(p, p->dstar_count, sizeof(u64) * cap))) return st;
+            if (!p->j_only && ((st = ensure(p, p->pc_col, sizeof(uint32_t) * cap)) || (st = ensure(p, p->pc_cnt, sizeof(u64) * cap)) ||
+                               (st = ensure(p, p->dstar_col, sizeof(uint32_t) * cap)) ||
+                               (st = ensure(p, p->dstar_count, sizeof(u64) * cap))))
+                return st;
             // a captured pass starts from a cleared summary, and its path count runs once
             if (!cap_mode && (st = check_cuda(p, cudaMemsetAsync(ctr, 0, sizeof(u64) * PC_SLOTS, s), "memset counters")))
                 return st;
@@ -956,6 +956,10 @@ msc_status run_path_count(Plan* p, cudaStream_t s) {
                     continue;
                 }
                 p->dp_pool_cap = int64_t(pool_used);
+                if (p->j_only)  // the D* that is there stays
+                    return p->hsum->dp_junctions_done == u64(njcap)
+                               ? MSC_OK
+                               : fail(p, MSC_ERR_INTERNAL, "internal: the waves did not reach every junction");
             }
             const u64* all_rows = &p->dsum()->counts[1];
             if ((st = check_cuda(p,

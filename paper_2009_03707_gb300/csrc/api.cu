@@ -31,6 +31,9 @@ msc_status ensure(Plan* p, DeviceBuffer& b, size_t bytes) {
     if (p->fault_kind == 1 && ++p->alloc_calls == p->fault_at)
         return fail(p, MSC_ERR_OOM, "injected allocation failure (MSC_FAULT)");
     if (b.ptr) {
+        // a captured pass may hold this address (a stage run by itself can outgrow what it was captured
+        // with): it is captured again
+        if (p->graph_exec && !p->capturing) destroy_graph(p);
         cudaFree(b.ptr);
         p->live_bytes -= int64_t(b.bytes);
         b.ptr = nullptr;

@@ -371,7 +371,8 @@ msc_status build_minor_csr(Plan* p, cudaStream_t s) {
         scratch_off[w] = scratch_total;
         scratch_total += (row_scan_scratch_bytes(rows[w]) + 255) / 256 * 256;
     }
-    if ((st = ensure(p, p->minor_scan, scratch_total ? scratch_total : 1))) return st;
+    // not minor_scan, which the captured pass keeps pointers to and which must not grow between its replays
+    if ((st = ensure(p, p->minor_csr_scan, scratch_total ? scratch_total : 1))) return st;
     // per-row counts of A (n1 rows), B, B* (nj), D (n1), in that order
     if ((st = ensure(p, p->minor_rowcnt, sizeof(uint32_t) * size_t(2 * (n1 + nj) ? 2 * (n1 + nj) : 1)))) return st;
     CsrArgs ca{};
@@ -391,7 +392,7 @@ msc_status build_minor_csr(Plan* p, cudaStream_t s) {
         if ((st = ensure(p, p->minor_rowptr[w], sizeof(int64_t) * size_t(rows[w] + 1)))) return st;
         ca.rowptr[w] = static_cast<const int64_t*>(p->minor_rowptr[w].ptr);
         p->minor_rows[w] = rows[w];
-        auto* scratch = reinterpret_cast<unsigned long long*>(static_cast<char*>(p->minor_scan.ptr) + scratch_off[w]);
+        auto* scratch = reinterpret_cast<unsigned long long*>(static_cast<char*>(p->minor_csr_scan.ptr) + scratch_off[w]);
         if ((st = check_cuda(p,
                              row_scan(p, ca.cnt[w], nullptr, rows[w], static_cast<int64_t*>(p->minor_rowptr[w].ptr),
                                       scratch, s),

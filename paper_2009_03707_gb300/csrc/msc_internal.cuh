@@ -91,7 +91,7 @@ struct Plan {
     DeviceBuffer vmin, cmax, min_arcs, max_arcs, ext_lab_v, ext_lab_c;
     DeviceBuffer visited, reach_tmp, reach_masks, reach_qdown, reach_stamp, reach_queue, node_info;
     DeviceBuffer junc_bits, junc_prefix, junc_cells;
-    DeviceBuffer trace, trace_kinds, minor_rowcnt, minor_scan, minor_rowptr[4], minor_col[4], minor_mult[4];
+    DeviceBuffer trace, trace_kinds, minor_rowcnt, minor_scan, minor_csr_scan, minor_rowptr[4], minor_col[4], minor_mult[4];
     DeviceBuffer pc_rowstart, pc_rowlen, pc_big, pc_col, pc_cnt, pc_gk, pc_gv, pc_gocc;
     DeviceBuffer dstar_rowptr, dstar_col, dstar_count;
     DeviceBuffer csc_colptr, csc_row, csc_count, csc_work;  // D* by 2-saddle (transpose.cu)
@@ -110,7 +110,7 @@ struct Plan {
         DeviceBuffer* all[] = {&words, &status, &crit_bits, &crit_prefix, &scan_sums, &cells[0], &cells[1], &cells[2],
                                &cells[3], &vmin, &cmax, &min_arcs, &max_arcs, &ext_lab_v, &ext_lab_c, &visited, &reach_tmp, &reach_masks,
                                &reach_qdown, &reach_stamp, &reach_queue, &node_info, &junc_bits, &junc_prefix, &junc_cells, &trace, &trace_kinds,
-                               &minor_rowcnt, &minor_scan, &minor_rowptr[0], &minor_rowptr[1], &minor_rowptr[2],
+                               &minor_rowcnt, &minor_scan, &minor_csr_scan, &minor_rowptr[0], &minor_rowptr[1], &minor_rowptr[2],
                                &minor_rowptr[3], &minor_col[0], &minor_col[1], &minor_col[2], &minor_col[3],
                                &minor_mult[0], &minor_mult[1], &minor_mult[2], &minor_mult[3], &pc_rowstart, &pc_rowlen,
                                &pc_big, &pc_col, &pc_cnt, &pc_gk, &pc_gv, &pc_gocc, &dstar_rowptr, &dstar_col,

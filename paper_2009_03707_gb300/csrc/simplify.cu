@@ -30,7 +30,7 @@
 // Four launches a round, their counts on the device; the host looks once per BATCH rounds.  At the
 // end one gather makes the CSR, and one stable sort by round puts the cancellations in log order.
 // 256^3 GRF (6.0 M nodes, 40 M entries, 317 rounds, threshold 5 % of the range): 370 ms with every
-// round sweeping all nodes and rewriting the whole CSR (1.1 ms a round), 73 ms now: looks 37, updates 14,
+// round sweeping all nodes and rewriting the whole CSR (1.1 ms a round), 66 ms now: looks 28, updates 14,
 // the list 11, cancellations 6.
 #include <cooperative_groups.h>
 
@@ -336,6 +336,24 @@ __global__ void __launch_bounds__(THREADS) simp_wake(SimpArgs a, int slot, uint3
 // rows' lengths (a lane per row: 1.5 times as long on the late rounds of the 256^3 GRF, whose rows
 // reach 128 entries).
 constexpr int AHEAD = 4;
+// The lane with the greatest key among those that have one: of the smaller keys found together, the one
+// likely to be there longest, since arcs go in about the order of their keys (looks on the 256^3 GRF:
+// 35 ms with any of them, 28 ms so).
+template <unsigned L>
+__device__ __forceinline__ int greatest(const cg::thread_block_tile<L, cg::thread_block>& t, bool has, Key k) {
+    if (!has) k = Key{0, 0};
+    uint32_t lane = has ? t.thread_rank() + 1 : 0u;  // 0: no key
+#pragma unroll
+    for (unsigned o = L / 2; o; o >>= 1) {
+        const Key other{t.shfl_xor(k.hi, o), t.shfl_xor(k.lo, o)};
+        const uint32_t other_lane = t.shfl_xor(lane, o);
+        if (key_less(k, other) || (!key_less(other, k) && other_lane > lane)) {
+            k = other;
+            lane = other_lane;
+        }
+    }
+    return int(lane) - 1;
+}
 template <unsigned L>
 __device__ __forceinline__ bool look_around(const SimpArgs& a, const cg::thread_block_tile<L, cg::thread_block>& t,
                                             uint32_t p, uint32_t q, const Key& k, uint32_t* v_out, uint32_t* w_out) {
@@ -347,9 +365,11 @@ __device__ __forceinline__ bool look_around(const SimpArgs& a, const cg::thread_
     };
     for (uint32_t e = r; e - r < n; e += L) {
         const uint32_t v = neighbour(e);
-        const uint32_t less = t.ballot(v != NO_NODE && key_less(a.node[v].least, k));
-        if (less) {
-            *v_out = *w_out = t.shfl(v, __ffs(less) - 1);
+        Key kv = no_key();
+        if (v != NO_NODE) kv = a.node[v].least;
+        const bool less = key_less(kv, k);
+        if (t.any(less)) {
+            *v_out = *w_out = t.shfl(v, greatest(t, less, kv));
             return true;
         }
     }
@@ -367,6 +387,7 @@ __device__ __forceinline__ bool look_around(const SimpArgs& a, const cg::thread_
         first -= vr.len;
         for (uint32_t j0 = 0; j0 < total; j0 += L * AHEAD) {
             uint32_t w[AHEAD], hit = NO_NODE, hit_l = 0;
+            Key hit_k{0, 0};
             int own[AHEAD];
 #pragma unroll
             for (int i = 0; i < AHEAD; ++i) {
@@ -381,13 +402,16 @@ __device__ __forceinline__ bool look_around(const SimpArgs& a, const cg::thread_
             }
 #pragma unroll
             for (int i = 0; i < AHEAD; ++i)
-                if (w[i] != NO_NODE && key_less(a.node[w[i]].least, k)) {
-                    hit = w[i];
-                    hit_l = own[i];
+                if (w[i] != NO_NODE) {
+                    const Key kw = a.node[w[i]].least;
+                    if (key_less(kw, k) && !key_less(kw, hit_k)) {
+                        hit = w[i];
+                        hit_l = own[i];
+                        hit_k = kw;
+                    }
                 }
-            const uint32_t less = t.ballot(hit != NO_NODE);
-            if (less) {
-                const int l = __ffs(less) - 1;
+            if (t.any(hit != NO_NODE)) {
+                const int l = greatest(t, hit != NO_NODE, hit_k);
                 *w_out = t.shfl(hit, l);
                 *v_out = t.shfl(v, t.shfl(hit_l, l));
                 return true;
@@ -440,8 +464,9 @@ __device__ __forceinline__ void look_at_arcs(const SimpArgs& a, RoundCount* out,
     }
 }
 // Many looks are bound by how many are in flight (8 lanes each), few by how long the longest takes (a
-// whole warp each): late rounds of the 256^3 GRF have some 2500 looks of up to 1850 entries.
-constexpr unsigned int WIDE_LOOKS = 32768;
+// whole warp each): late rounds of the 256^3 GRF have some 2500 looks of up to 1850 entries (all looks:
+// 40, 37 and 35 ms with the line at 16, 32 and 64 thousand).
+constexpr unsigned int WIDE_LOOKS = 65536;
 __global__ void __launch_bounds__(THREADS) simp_look(SimpArgs a, int slot) {
     if (a.state->halted) return;
     RoundCount* out = &a.state->round[slot + 1];

@@ -22,14 +22,15 @@
 //    size (1..27 cells) and a warp runs as long as its largest, so the CTA first sizes every star
 //    and counting-sorts its vertices by size; warps then claim 32 consecutive stars at a time,
 //    largest first.
-//  * A second, bandwidth-bound kernel turns the finished words into per-slot critical bitmaps:
-//    one warp ballot per slot gives 32 vertices' bits -- the input of the ordered compaction.
+//  * A second kernel turns the finished words into per-slot critical bitmaps, the input of the
+//    ordered compaction (word_bitmaps.cuh).
 #include <map>
 #include <mutex>
 #include <tuple>
 
 #include "lower_star.cuh"
 #include "msc_internal.cuh"
+#include "word_bitmaps.cuh"
 
 namespace msc {
 
@@ -242,41 +243,6 @@ __global__ void __launch_bounds__(THREADS, 65536 / (64 * THREADS)) gradient_kern
     }
 }
 
-// Per-slot critical bitmaps from finished words: one warp per CB_WORDS row words of 32 vertices,
-// their loads issued together.
-constexpr int CB_WORDS = 4;
-__global__ void __launch_bounds__(256) critical_bitmaps(Geom g, const uint32_t* __restrict__ words,
-                                                        uint32_t* __restrict__ crit_bits) {
-    const uint32_t nrw = uint32_t(g.nz) * uint32_t(g.ny) * uint32_t(g.W);  // < 2^28 row words
-    const uint32_t w0 = ((blockIdx.x * blockDim.x + threadIdx.x) >> 5) * CB_WORDS;
-    const int lane = threadIdx.x & 31;
-    if (w0 >= nrw) return;  // warp-uniform
-    uint32_t word[CB_WORDS];
-    int w[CB_WORDS], y[CB_WORDS], z[CB_WORDS];
-#pragma unroll
-    for (int u = 0; u < CB_WORDS; ++u) {
-        const uint32_t wid = min(w0 + u, nrw - 1);
-        const uint32_t q = g.div_W.div(wid);
-        w[u] = int(wid - q * uint32_t(g.W));
-        z[u] = int(g.div_ny.div(q));
-        y[u] = int(q - uint32_t(z[u]) * uint32_t(g.ny));
-        const int x = w[u] * 32 + lane;
-        word[u] = x < g.nx ? words[uint32_t(x) + uint32_t(g.nx) * (uint32_t(y[u]) + uint32_t(g.ny) * uint32_t(z[u]))]
-                           : 0x00FFFFFFu;  // all codes 7: no cell
-    }
-#pragma unroll
-    for (int u = 0; u < CB_WORDS; ++u) {
-        if (w0 + u >= nrw) break;  // warp-uniform
-        uint32_t mine = 0;
-#pragma unroll
-        for (int s = 0; s < 8; ++s) {
-            const uint32_t bits = __ballot_sync(0xFFFFFFFFu, slot_code(word[u], s) == 0);
-            if (lane == s) mine = bits;
-        }
-        if (lane < 8) crit_bits[g.slot_word(lane, z[u], y[u], w[u])] = mine;
-    }
-}
-
 // Zeroes the words that the lower-star kernel finishes with atomicOr: those on the + faces of its
 // tiles (x = 31 mod 32, y = TY-1 mod TY, z = TZ-1 mod TZ), which receive codes from the next tiles'
 // stars.  Every other word gets one plain store, so it needs no zeroing.  A warp per (y, z) row:
@@ -344,7 +310,7 @@ cudaError_t launch_words(int v, const Geom& g, const float* d_field, uint32_t* w
     }
 }
 
-cudaError_t launch_gradient(int v, const Geom& g, const float* d_field, uint32_t* words, uint32_t* crit_bits,
+cudaError_t launch_gradient(int v, const Geom& g, const float* d_field, uint32_t* words, const WordBitmaps& maps,
                             uint32_t* status, cudaStream_t s, const Plan* p = nullptr) {
     cudaError_t e = launch_zero_faces(v, g, words, s, p && p->capturing ? p->dsum() : nullptr);
     if (e != cudaSuccess) return e;
@@ -362,9 +328,8 @@ cudaError_t launch_gradient(int v, const Geom& g, const float* d_field, uint32_t
     }
     if (p) record_event(p, p->gev1, s);
     if (e != cudaSuccess) return e;
-    const int64_t warps = (int64_t(g.nz) * g.ny * g.W + CB_WORDS - 1) / CB_WORDS;
-    critical_bitmaps<<<int((warps * 32 + 255) / 256), 256, 0, s>>>(g, words, crit_bits);
-    return cudaGetLastError();
+    return p && p->capturing ? launch_word_bitmaps<true, true>(g, maps, p->num_sms, s)
+                             : launch_word_bitmaps<true, false>(g, maps, p ? p->num_sms : 0, s);
 }
 
 // Autotuning: the tile variant that computes this grid's words fastest on this device, timed on
@@ -429,9 +394,9 @@ msc_status run_gradient(Plan* p, const float* d_field, cudaStream_t s) {
     const int v = std::max(0, p->grad_variant);
     p->stats.gradient_tile = VARIANTS[v].ty | (VARIANTS[v].tz << 8) | (int64_t(VARIANTS[v].threads) << 16);
     launched(p, 3);
-    return check_cuda(p,
-                      launch_gradient(v, g, d_field, static_cast<uint32_t*>(p->words.ptr),
-                                      static_cast<uint32_t*>(p->crit_bits.ptr), p->status_word(), s, p),
+    // a captured pass makes the reachability's bitmaps from the same reading of the words
+    if (p->capturing && (st = ensure_reach_maps(p))) return st;
+    return check_cuda(p, launch_gradient(v, g, d_field, static_cast<uint32_t*>(p->words.ptr), maps_of(p), p->status_word(), s, p),
                       "gradient launch");
 }
 
@@ -445,7 +410,7 @@ cudaError_t load_gradient_raw() {
     if (e == cudaSuccess)
         e = cudaFuncSetAttribute(gradient_kernel<8, 8, 512>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                  int(sizeof(Shared<8, 8, 512>)));
-    if (e == cudaSuccess) e = cudaFuncGetAttributes(&a, critical_bitmaps);
+    if (e == cudaSuccess) e = cudaFuncGetAttributes(&a, word_bitmaps<true, false>);
     return e;
 }
 
@@ -453,7 +418,10 @@ cudaError_t load_gradient_raw() {
 // no-allocation entry point, static_entry.cu).
 cudaError_t launch_gradient_raw(const Geom& g, const float* d_field, uint32_t* words, uint32_t* crit_bits,
                                 uint32_t* status, cudaStream_t s) {
-    return launch_gradient(0, g, d_field, words, crit_bits, status, s);
+    WordBitmaps maps{};
+    maps.words = words;
+    maps.crit_bits = crit_bits;
+    return launch_gradient(0, g, d_field, words, maps, status, s);
 }
 
 }  // namespace msc

@@ -264,6 +264,9 @@ msc_status build_arc_geometry(Plan* p, cudaStream_t s);   // cells along the sad
 msc_status build_ss_geometry(Plan* p, cudaStream_t s);    // cells along the saddle-saddle arcs of count 1 (needs J; syncs)
 msc_status run_simplify(Plan* p, const float* d_field, double threshold, cudaStream_t s);  // (on request; syncs)
 msc_status run_junction_dp(Plan* p, cudaStream_t s, uint64_t pool_cap, uint64_t out_cap);
+msc_status ensure_reach_maps(Plan* p);  // the buffers of the reachability's bitmaps (reach.cu)
+struct WordBitmaps;
+WordBitmaps maps_of(const Plan* p);
 int grid_cap(const Plan* p, int64_t threads, int block, int per_sm = 8);  // grid for a count-bounded loop
 
 }  // namespace msc

@@ -38,6 +38,7 @@
 
 #include "dag.cuh"
 #include "scan.cuh"
+#include "word_bitmaps.cuh"
 
 namespace cg = cooperative_groups;
 
@@ -46,8 +47,6 @@ namespace msc {
 namespace {
 
 constexpr int THREADS = 256;
-
-__device__ __forceinline__ int other_axis(int a, int j) { return j == 0 ? (a == 0 ? 1 : 0) : (a == 2 ? 1 : 2); }
 
 // Word addressing of the bitmaps, per thread: the 1-cell row layout is
 //   edge_word(z, c, y, b, w) = z*sz + y*sy + off[axis] + w   (sz = 4 ny W, sy = 2 W),
@@ -113,81 +112,6 @@ __device__ __forceinline__ uint32_t pull(uint32_t m, const uint32_t* __restrict_
                        reach_row<B, ux - back * bx, uy - back * by, uz - back * bz>(R, r) |
                        reach_row<B, -back * bx, -back * by, -back * bz>(R, r);
     return m & p;
-}
-
-// Per vertex-row word: for each axis the four masks of 1-cells paired with the quad on the - / +
-// side along the first / second other axis, R_0 = the 1-saddles, and for each quad orientation (by
-// its even axis k) the bitmap of quads that are critical or paired with a facet (the quads that
-// give an out-edge to every other facet).  A warp takes `chunk` (4..32, a multiple of RI_WORDS)
-// consecutive row words: it builds each word's bitmaps with one ballot apiece (a lane per x),
-// RI_WORDS words' loads issued together, keeps word u's bitmaps in lane u, and then writes all of
-// them with one store per array.  Large grids take chunks of 32 (the stores fully coalesced), small
-// ones smaller chunks so that enough warps share the work.
-constexpr int RI_WORDS = 4;
-__global__ void __launch_bounds__(THREADS) reach_init(Geom g, const uint32_t* __restrict__ words,
-                                                      uint4* __restrict__ masks, uint32_t* __restrict__ R0,
-                                                      uint32_t* __restrict__ R1, uint32_t* __restrict__ qdown,
-                                                      uint32_t* __restrict__ stamp, int chunk) {
-    const int lane = threadIdx.x & 31;
-    const int64_t nrw = int64_t(g.nz) * g.ny * g.W;
-    const int64_t step = ((int64_t(gridDim.x) * THREADS) >> 5) * chunk;
-    for (int64_t t0 = ((int64_t(blockIdx.x) * THREADS + threadIdx.x) >> 5) * chunk; t0 < nrw; t0 += step) {
-        uint4 m[3];
-        uint32_t crit[3], qd[3];
-        for (int u0 = 0; u0 < chunk && t0 + u0 < nrw; u0 += RI_WORDS) {  // warp-uniform
-            uint32_t words_of[RI_WORDS];
-#pragma unroll
-            for (int v = 0; v < RI_WORDS; ++v) {
-                const Rows r(g, min(t0 + u0 + v, nrw - 1));
-                const int x = r.w * 32 + lane;
-                words_of[v] = x < g.nx ? words[vid32(g, x, r.y, r.z)] : 0x00FFFFFFu;  // all codes 7 off-grid
-            }
-#pragma unroll
-            for (int v = 0; v < RI_WORDS; ++v) {
-                const bool mine = lane == u0 + v;  // this lane keeps word u0 + v's bitmaps
-                const uint32_t word = words_of[v];
-#pragma unroll
-                for (int a = 0; a < 3; ++a) {
-                    const uint32_t code = slot_code(word, 1 << a);
-                    const int k = int(code - 1) >> 1;  // axis of the partner (code 1..6)
-                    const bool quad = code >= 1 && code <= 6 && k != a;
-                    const int sel = quad ? 2 * (k == other_axis(a, 0) ? 0 : 1) + int(!(code & 1u)) : -1;  // odd: - side
-                    const uint32_t m0 = __ballot_sync(0xFFFFFFFFu, sel == 0), m1 = __ballot_sync(0xFFFFFFFFu, sel == 1);
-                    const uint32_t m2 = __ballot_sync(0xFFFFFFFFu, sel == 2), m3 = __ballot_sync(0xFFFFFFFFu, sel == 3);
-                    const uint32_t c0 = __ballot_sync(0xFFFFFFFFu, code == 0);
-                    if (mine) {
-                        m[a] = make_uint4(m0, m1, m2, m3);
-                        crit[a] = c0;
-                    }
-                }
-#pragma unroll
-                for (int k = 0; k < 3; ++k) {
-                    const uint32_t code = slot_code(word, 7 ^ (1 << k));
-                    const bool down = code == 0 || (code <= 6 && (int(code - 1) >> 1) != k);
-                    const uint32_t q = __ballot_sync(0xFFFFFFFFu, down);
-                    if (mine) qd[k] = q;
-                }
-            }
-        }
-        const int64_t t = t0 + lane;
-        if (lane < chunk && t < nrw) {
-            const Rows r(g, t);
-            const int e0 = r.edge<0>(0, 0), e1 = r.edge<1>(0, 0), e2 = r.edge<2>(0, 0);
-            masks[e0] = m[0];
-            masks[e1] = m[1];
-            masks[e2] = m[2];
-            R0[e0] = crit[0];
-            R0[e1] = crit[1];
-            R0[e2] = crit[2];
-#pragma unroll
-            for (int k = 0; k < 3; ++k) qdown[k * r.qplane + r.qbase] = qd[k];
-            if (r.w == 0) stamp[r.z * r.ny + r.y] = 1;  // every row is new at the start
-            // the unused slot of the 1-cell layout stays empty in both buffers
-            masks[e2 + r.W] = make_uint4(0, 0, 0, 0);
-            R0[e2 + r.W] = 0;
-            R1[e2 + r.W] = 0;
-        }
-    }
 }
 
 template <int A>
@@ -796,29 +720,40 @@ msc_status launch_tail(Plan* p, cudaStream_t s, const PushArgs& a, int all) {
 
 }  // namespace
 
+msc_status ensure_reach_maps(Plan* p) {
+    const Geom& g = p->g;
+    const size_t nw = size_t(g.edge_words()), nrw = size_t(g.nz) * size_t(g.ny) * size_t(g.W);
+    msc_status st;
+    if ((st = ensure(p, p->visited, sizeof(uint32_t) * nw))) return st;
+    if ((st = ensure(p, p->reach_tmp, sizeof(uint32_t) * nw))) return st;
+    if ((st = ensure(p, p->reach_masks, sizeof(uint4) * nw))) return st;
+    if ((st = ensure(p, p->reach_qdown, sizeof(uint32_t) * 3 * nrw))) return st;
+    return ensure(p, p->reach_stamp, sizeof(uint32_t) * size_t(g.nz) * size_t(g.ny));
+}
+
+WordBitmaps maps_of(const Plan* p) {
+    return WordBitmaps{static_cast<const uint32_t*>(p->words.ptr),     static_cast<uint32_t*>(p->crit_bits.ptr),
+                       static_cast<uint4*>(p->reach_masks.ptr),        static_cast<uint32_t*>(p->visited.ptr),
+                       static_cast<uint32_t*>(p->reach_tmp.ptr),       static_cast<uint32_t*>(p->reach_qdown.ptr),
+                       static_cast<uint32_t*>(p->reach_stamp.ptr)};
+}
+
 msc_status run_reachability(Plan* p, cudaStream_t s) {
     const Geom& g = p->g;
     msc_status st;
-    const int64_t nw = g.edge_words();
     const int64_t nrw = int64_t(g.nz) * g.ny * g.W;  // vertex-row words
-    if ((st = ensure(p, p->visited, sizeof(uint32_t) * size_t(nw)))) return st;
-    if ((st = ensure(p, p->reach_tmp, sizeof(uint32_t) * size_t(nw)))) return st;
-    if ((st = ensure(p, p->reach_masks, sizeof(uint4) * size_t(nw)))) return st;
-    if ((st = ensure(p, p->reach_qdown, sizeof(uint32_t) * 3 * size_t(nrw)))) return st;
-    if ((st = ensure(p, p->reach_stamp, sizeof(uint32_t) * size_t(g.nz) * size_t(g.ny)))) return st;
+    if ((st = ensure_reach_maps(p))) return st;
     auto* masks = static_cast<uint4*>(p->reach_masks.ptr);
     auto* stamp = static_cast<uint32_t*>(p->reach_stamp.ptr);
     uint32_t* A = static_cast<uint32_t*>(p->visited.ptr);
     uint32_t* B = static_cast<uint32_t*>(p->reach_tmp.ptr);
-    // row words per warp: 32 when every SM still gets 32 warps' worth, else fewer (at least 4)
-    int chunk = 32;
-    while (chunk > RI_WORDS && nrw < int64_t(chunk) * 32 * std::max(1, p->num_sms)) chunk >>= 1;
-    reach_init<<<grid_for(p, (nrw + chunk - 1) / chunk * 32), THREADS, 0, s>>>(
-        g, static_cast<const uint32_t*>(p->words.ptr), masks, A, B, static_cast<uint32_t*>(p->reach_qdown.ptr), stamp,
-        chunk);
+    if (!p->capturing) {  // a captured pass made them with the critical bitmaps
+        if ((st = check_cuda(p, launch_word_bitmaps<false, true>(g, maps_of(p), p->num_sms, s), "word_bitmaps launch"))) return st;
+        launched(p);
+    }
     reach_start<<<1, 1, 0, s>>>(p->dsum());
-    launched(p, 2);
-    if ((st = check_cuda(p, cudaGetLastError(), "reach_init launch"))) return st;
+    launched(p);
+    if ((st = check_cuda(p, cudaGetLastError(), "reach_start launch"))) return st;
     // sweep grid: at most 4 tiles per CTA and at least one resident wave (4 CTAs per SM).  Fewer,
     // longer CTAs would cost little alone but leave long tails when other passes share the device.
     const int64_t tiles = (nrw + THREADS - 1) / THREADS;

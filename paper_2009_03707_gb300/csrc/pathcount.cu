@@ -105,7 +105,7 @@ __device__ __forceinline__ uint4 trace_of(const PcArgs& a, int64_t src) {
 // junction's trace and adds each traced path to the owning row's next frontier or D* table
 // with shared-memory atomics.  So a lane's work does not depend on its own row's size, and
 // every per-row loop is a fixed, unrolled one.  A row whose table fills up, or whose counts
-// outgrow 32 bits, is deferred intact to the next tier (tier 0b, the same kernel with larger
+// outgrow 32 bits, is deferred intact to the next tier (tier 0b, eight lanes a row with larger
 // tables, then the uint64 warp tier).
 //
 // Packed tables (PK): a slot is one word, key << 8 | count, for keys below 2^24 - 1 (then a

@@ -43,13 +43,6 @@ using star::pdx;
 using star::pdy;
 using star::pdz;
 
-// Monotone map float -> uint32 (IEEE order; -0 and +0 map to the same key).
-__device__ __forceinline__ uint32_t order_key(float f) {
-    uint32_t u = __float_as_uint(f);
-    if ((u & 0x7fffffffu) == 0) u = 0;
-    return (u & 0x80000000u) ? ~u : (u | 0x80000000u);
-}
-
 // The owned tile is TX x TY x TZ vertices, run by THREADS threads (a tuning choice: every
 // variant computes the same words).
 template <int TY, int TZ, int THREADS>
@@ -115,7 +108,7 @@ __global__ void __launch_bounds__(THREADS, 65536 / (64 * THREADS)) gradient_kern
         const int gx = x0 - 1 + fx, gy = y0 - 1 + fy, gz = z0 - 1 + fz;
         const bool in = gx >= 0 && gy >= 0 && gz >= 0 && gx < g.nx && gy < g.ny && gz < g.nz;
         saw_nan |= in && isnan(v[k]);
-        sh.fkey[fz][fy][fx] = in ? order_key(v[k]) : OUTSIDE_KEY;
+        sh.fkey[fz][fy][fx] = in ? star::order_key_of_bits(__float_as_uint(v[k])) : OUTSIDE_KEY;
     }
     if (saw_nan) atomicOr(status, ST_NAN);
     __syncthreads();

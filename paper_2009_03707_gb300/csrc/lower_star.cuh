@@ -105,6 +105,16 @@ __host__ __device__ inline uint32_t cell_vertices(int p) {
     return xs & ys & zs & ~(1u << CENTER);
 }
 
+// Monotone map of a float's bits to uint32 (IEEE order; -0 and +0 map to the same key).  Every NaN above
+// infinity gets one key, just above infinity's: a field with a NaN is rejected, but the kernel has run on it
+// by then, and a NaN's own bits reach up to the key of an off-grid vertex and to the padding words of
+// rank_cell_keys, which have to stay above every key of the grid.
+constexpr uint32_t NAN_KEY = 0xFF800001u;
+__host__ __device__ __forceinline__ uint32_t order_key_of_bits(uint32_t u) {
+    if ((u & 0x7FFFFFFFu) == 0) u = 0;
+    return (u & 0x80000000u) ? ~u : MSC_UMIN(u | 0x80000000u, NAN_KEY);
+}
+
 // Per-position masks, tabulated once per CTA (shared memory on the device): a 27-entry table of
 // 32-bit words sits in 27 distinct banks, so divergent lanes read it without conflicts.  off[p]
 // is where the key of the vertex at position p sits relative to the key of x in the caller's
@@ -293,7 +303,8 @@ __host__ __device__ constexpr int star_pos(int i) { return i < CENTER ? i : i + 
 // center points at x's key; ROW and PLANE are the key array's strides along y and z, off the same as
 // an offset per position (Tables::off).
 //  1. Each vertex of L(x) gets the 32-bit word (key with its low 5 bits cleared) | position, and
-//     each other position a padding word above all of them (spaced 32 apart).  A sorting
+//     each other position a padding word above all of them (spaced 32 apart; no key exceeds
+//     NAN_KEY, so no word agrees with a padding word above bit 4).  A sorting
 //     network orders the 26 words; these words order two vertices exactly as (key, position)
 //     does unless their keys agree in all but the low 5 bits and those are the other way round
 //     from the positions.  Two such vertices end up adjacent, or with others like them between,
@@ -309,6 +320,7 @@ __host__ __device__ constexpr int star_pos(int i) { return i < CENTER ? i : i + 
 template <int ROW, int PLANE, class Scratch>
 __host__ __device__ __forceinline__ bool rank_cell_keys(const uint32_t inL, const uint32_t* center, const int* off,
                                                         Scratch&& K) {
+    static_assert((NAN_KEY | 31u) < 0xFFFFFFFFu - 32u * 25u, "the padding words lie above every key");
     uint32_t v[26];
 #pragma unroll
     for (int i = 0; i < 26; ++i) {

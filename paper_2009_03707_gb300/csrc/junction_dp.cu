@@ -75,10 +75,10 @@ struct DpArgs {
     uint32_t* status;
 };
 
-// The pass's counts; false (do nothing) when the pass is to be rerun.
+// The pass's counts; false (do nothing) when the pass is to be rerun.  Called by whole blocks.
 __device__ __forceinline__ bool counts_of(const DpArgs& a, int64_t& n1, int64_t& nj) {
     const u64 x = *a.n1_dev, y = *a.nj_dev;
-    if (pass_retrying(a.status) || !count_fits(a.status, x, a.cap1) || !count_fits(a.status, y, a.capj)) return false;
+    if (block_retrying(a.status) || !count_fits(a.status, x, a.cap1) || !count_fits(a.status, y, a.capj)) return false;
     n1 = int64_t(x);
     nj = int64_t(y);
     return true;

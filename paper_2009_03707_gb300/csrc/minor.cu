@@ -97,7 +97,7 @@ __device__ __forceinline__ uint32_t distinct_count(const uint32_t rank[4], const
 // (1200 warp instructions per 32 sources, 71 % of the issue rate), 0.489 ms.
 __global__ void __launch_bounds__(THREADS, 6) trace_kernel(TraceArgs a) {
     const unsigned long long n1 = *a.n1_dev, nj = *a.nj_dev;
-    if (pass_retrying(a.status) || !count_fits(a.status, n1, a.cap1) || !count_fits(a.status, nj, a.capj)) return;
+    if (block_retrying(a.status) || !count_fits(a.status, n1, a.cap1) || !count_fits(a.status, nj, a.capj)) return;
     const Geom& g = a.g;
     const uint32_t nx = uint32_t(g.nx), ny = uint32_t(g.ny), nz = uint32_t(g.nz), W = uint32_t(g.W);
     const uint32_t N1 = uint32_t(n1), NS = uint32_t(n1 + nj);

@@ -32,6 +32,10 @@ enum StatusBit : uint32_t {
 __device__ __forceinline__ bool pass_retrying(const uint32_t* status) {
     return (*reinterpret_cast<const volatile uint32_t*>(status) & ST_RETRY) != 0;
 }
+// pass_retrying for a block whose threads or warps work together: one answer for all of them, so every thread
+// of the block calls it.  Another block, or the extremum branch beside this one, may raise ST_RETRY between two
+// warps' reads, and what is left of a block would go on with shared counts that nobody has set.
+__device__ __forceinline__ bool block_retrying(const uint32_t* status) { return __syncthreads_or(pass_retrying(status)) != 0; }
 __device__ __forceinline__ bool count_fits(uint32_t* status, unsigned long long n, int64_t cap) {
     if (n <= (unsigned long long)cap) return true;
     if (threadIdx.x == 0) atomicOr(status, ST_RETRY);

@@ -81,10 +81,10 @@ struct PcArgs {
 __device__ __forceinline__ int64_t row_of(const PcArgs& a, int64_t i) { return a.rows ? int64_t(a.rows[i]) : i; }
 
 // The counts a launch works on, read on the device (they are produced earlier in the same pass);
-// false (do nothing) when the pass is to be rerun.
+// false (do nothing) when the pass is to be rerun.  Called by whole blocks.
 __device__ __forceinline__ bool resolve(PcArgs& a) {
     const unsigned long long n1 = *a.n1_dev, nj = *a.nj_dev;
-    if (pass_retrying(a.status) || !count_fits(a.status, n1, a.n1_cap) || !count_fits(a.status, nj, a.nj_cap))
+    if (block_retrying(a.status) || !count_fits(a.status, n1, a.n1_cap) || !count_fits(a.status, nj, a.nj_cap))
         return false;
     a.n1 = int64_t(n1);
     a.nrows = int64_t(min(*a.nrows_dev, n1));
@@ -876,7 +876,7 @@ __global__ void gather_rows(const unsigned long long* n1_dev, int64_t cap, const
                             const int64_t* __restrict__ rowptr, const uint32_t* __restrict__ in_col,
                             const u64* __restrict__ in_cnt, uint32_t* __restrict__ col, u64* __restrict__ cnt,
                             uint32_t* status) {
-    if (pass_retrying(status) || !count_fits(status, *n1_dev, cap)) return;
+    if (block_retrying(status) || !count_fits(status, *n1_dev, cap)) return;
     const int64_t n1 = int64_t(*n1_dev);
     const int lane = threadIdx.x & 31;
     const int64_t nwarps = (int64_t(gridDim.x) * blockDim.x) >> 5;

@@ -332,7 +332,7 @@ __global__ void __launch_bounds__(THREADS) reach_frontier(PushArgs a, const uint
 // One pushed level by the whole device: the queue `from` (count push_count[in]) to the other one (count
 // push_count[out]).
 __global__ void __launch_bounds__(THREADS) reach_push(PushArgs a, Summary* sum, int from, int in, int out) {
-    if (pass_retrying(a.status)) return;
+    if (block_retrying(a.status)) return;
     const uint32_t n = sum->push_count[in];
     __shared__ uint32_t base;
     for (uint64_t b = uint64_t(blockIdx.x) * THREADS; b < n; b += uint64_t(gridDim.x) * THREADS) {

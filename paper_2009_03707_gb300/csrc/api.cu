@@ -27,13 +27,14 @@ msc_status check_cuda(Plan* p, cudaError_t e, const char* what) {
 
 msc_status ensure(Plan* p, DeviceBuffer& b, size_t bytes) {
     if (bytes == 0) bytes = 16;
+    if (p->capturing) b.captured = true;
     if (b.ptr && b.bytes >= bytes) return MSC_OK;
-    if (p->fault_kind == 1 && ++p->alloc_calls == p->fault_at)
+    if (p->fault_kind == 1 && ++p->fault_calls == p->fault_at)
         return fail(p, MSC_ERR_OOM, "injected allocation failure (MSC_FAULT)");
     if (b.ptr) {
-        // a captured pass may hold this address (a stage run by itself can outgrow what it was captured
-        // with): it is captured again
-        if (p->graph_exec && !p->capturing) destroy_graph(p);
+        // a captured pass that holds this address (a stage run by itself can outgrow what it was captured
+        // with) is captured again; the buffers of what is asked for after a pass are in no capture
+        if (b.captured && p->graph_exec && !p->capturing) destroy_graph(p);
         cudaFree(b.ptr);
         p->live_bytes -= int64_t(b.bytes);
         b.ptr = nullptr;
@@ -153,13 +154,16 @@ msc_status run_loop(Plan* p, cudaStream_t s, int which, int body_launches,
                       "capture dependencies");
 }
 
-// MSC_FAULT = alloc@k | timeout | overflow: host-side fault injection for tests.
+// MSC_FAULT = alloc@k | capture@k | timeout | overflow (the k-th growth of a buffer, the k-th capture): host-side fault injection for tests.
 void read_fault(Plan* p) {
     const char* f = std::getenv("MSC_FAULT");
     if (!f) return;
     if (!std::strncmp(f, "alloc@", 6)) {
         p->fault_kind = 1;
         p->fault_at = std::atoll(f + 6);
+    } else if (!std::strncmp(f, "capture@", 8)) {
+        p->fault_kind = 4;
+        p->fault_at = std::atoll(f + 8);
     } else if (!std::strcmp(f, "timeout")) {
         p->fault_kind = 2;
     } else if (!std::strcmp(f, "overflow")) {
@@ -313,6 +317,7 @@ void destroy_graph(Plan* p) {
     p->graph_exec = nullptr;
     p->graph = nullptr;
     p->graph_field = nullptr;
+    p->for_each_buffer([](DeviceBuffer& b) { b.captured = false; });
     ++p->capture_epoch;
 }
 
@@ -321,6 +326,8 @@ void destroy_graph(Plan* p) {
 // and is discarded; the second records the graph that is replayed.
 msc_status capture_graph(Plan* p, const float* d_field) {
     destroy_graph(p);
+    if (p->fault_kind == 4 && ++p->fault_calls == p->fault_at)
+        return fail(p, MSC_ERR_CUDA, "injected capture failure (MSC_FAULT)");
     msc_status st = MSC_OK;
     const bool branch = !(p->opts.flags & MSC_FLAG_SERIAL_PASS);
     for (int pass = 0; pass < 2; ++pass) {

@@ -76,6 +76,7 @@ struct Summary {
 struct DeviceBuffer {
     void* ptr = nullptr;
     size_t bytes = 0;
+    bool captured = false;  // the plan's captured pass holds its address
 };
 
 struct Plan {
@@ -195,8 +196,8 @@ struct Plan {
     cudaStream_t pending_stream = nullptr;
     // host-side fault injection (MSC_FAULT, read at plan creation; tests only): the failure is
     // made on the host -- a faked allocation failure, or a status bit raised as a kernel would
-    int fault_kind = 0;  // 0 none, 1 alloc, 2 timeout (reachability), 3 overflow (path count)
-    int64_t fault_at = 0, alloc_calls = 0;
+    int fault_kind = 0;  // 0 none, 1 alloc, 2 timeout (reachability), 3 overflow (path count), 4 capture
+    int64_t fault_at = 0, fault_calls = 0;
 };
 
 // The trace of the DAG minor (minor.cu): for every 1-saddle (ranks 0..n1-1) then every junction
@@ -250,7 +251,7 @@ msc_status finish_replay(Plan* p, cudaStream_t s);
 msc_status compute_synchronised(Plan* p, const float* d_field, cudaStream_t s);
 msc_status bind_device(Plan* p);
 void invalidate(Plan* p);
-inline bool graphs_enabled(const Plan* p) { return !(p->opts.flags & MSC_FLAG_NO_GRAPH) && p->fault_kind == 0; }
+inline bool graphs_enabled(const Plan* p) { return !(p->opts.flags & MSC_FLAG_NO_GRAPH) && (p->fault_kind == 0 || p->fault_kind == 4); }
 msc_status read_summary(Plan* p, cudaStream_t s);       // syncs; copies the summary to p->hsum
 
 // Stage launchers

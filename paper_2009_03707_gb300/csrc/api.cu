@@ -154,7 +154,8 @@ msc_status run_loop(Plan* p, cudaStream_t s, int which, int body_launches,
                       "capture dependencies");
 }
 
-// MSC_FAULT = alloc@k | capture@k | timeout | overflow (the k-th growth of a buffer, the k-th capture): host-side fault injection for tests.
+// MSC_FAULT = alloc@k | capture@k | queue@n | timeout | overflow (the k-th growth of a buffer or the k-th capture
+// fails; the reachability's queues have room for n cells): host-side fault injection for tests.
 void read_fault(Plan* p) {
     const char* f = std::getenv("MSC_FAULT");
     if (!f) return;
@@ -164,6 +165,9 @@ void read_fault(Plan* p) {
     } else if (!std::strncmp(f, "capture@", 8)) {
         p->fault_kind = 4;
         p->fault_at = std::atoll(f + 8);
+    } else if (!std::strncmp(f, "queue@", 6)) {
+        p->fault_kind = 5;
+        p->fault_at = std::atoll(f + 6);
     } else if (!std::strcmp(f, "timeout")) {
         p->fault_kind = 2;
     } else if (!std::strcmp(f, "overflow")) {

@@ -160,7 +160,7 @@ struct Plan {
     int64_t capture_epoch = 0;        // bumped whenever the plan's graph is captured or dropped
     int tail_cluster = 0;             // blocks of the reachability's last-levels cluster (0: not asked yet)
     int64_t reach_iters = 1;          // sweep iterations of the last synchronised pass (two sweeps each)
-    bool reach_sweeps_only = false;   // a level outgrew the push queue on this plan
+    bool reach_sweeps_only = false;   // a level outgrew the push queue in the last synchronised pass
     int grad_variant = -1;            // gradient tile variant (-1: not tuned yet)
 
     int64_t counts[4] = {0, 0, 0, 0};
@@ -196,7 +196,7 @@ struct Plan {
     cudaStream_t pending_stream = nullptr;
     // host-side fault injection (MSC_FAULT, read at plan creation; tests only): the failure is
     // made on the host -- a faked allocation failure, or a status bit raised as a kernel would
-    int fault_kind = 0;  // 0 none, 1 alloc, 2 timeout (reachability), 3 overflow (path count), 4 capture
+    int fault_kind = 0;  // 0 none, 1 alloc, 2 timeout (reachability), 3 overflow (path count), 4 capture, 5 a small queue (reachability)
     int64_t fault_at = 0, fault_calls = 0;
 };
 
@@ -251,7 +251,7 @@ msc_status finish_replay(Plan* p, cudaStream_t s);
 msc_status compute_synchronised(Plan* p, const float* d_field, cudaStream_t s);
 msc_status bind_device(Plan* p);
 void invalidate(Plan* p);
-inline bool graphs_enabled(const Plan* p) { return !(p->opts.flags & MSC_FLAG_NO_GRAPH) && (p->fault_kind == 0 || p->fault_kind == 4); }
+inline bool graphs_enabled(const Plan* p) { return !(p->opts.flags & MSC_FLAG_NO_GRAPH) && (p->fault_kind == 0 || p->fault_kind >= 4); }
 msc_status read_summary(Plan* p, cudaStream_t s);       // syncs; copies the summary to p->hsum
 
 // Stage launchers

@@ -414,6 +414,7 @@ __global__ void __launch_bounds__(TAIL_THREADS, 1) reach_tail(PushArgs a, Summar
         if (threadIdx.x == 0) level_n = shared_counts[2];
         __syncthreads();
         n = level_n;
+        if (n > a.cap && threadIdx.x == 0) atomicOr(a.status, ST_RETRY);
     }
     // level k reads queue k & 1 and counts its new cells in counts[k % 3]; counts[(k + 1) % 3], last read
     // before level k - 1 began, is cleared for the next level
@@ -439,11 +440,13 @@ __global__ void __launch_bounds__(TAIL_THREADS, 1) reach_tail(PushArgs a, Summar
                         n = 0;
                     }
                     if (!n) break;
+                    // a level that goes on here is whole in shared memory, whatever the queues' room
                     uint32_t* to = n > TAIL_THREADS ? a.queue[k & 1] : alone;
-                    if (n > a.cap && threadIdx.x == 0) atomicOr(a.status, ST_RETRY);
+                    const uint32_t room = n > TAIL_THREADS ? a.cap : uint32_t(TAIL_THREADS);
+                    if (n > room && threadIdx.x == 0) atomicOr(a.status, ST_RETRY);
 #pragma unroll
                     for (int j = 0; j < 4; ++j)
-                        if (j < m && at + j < a.cap) to[at + j] = next[j];
+                        if (j < m && at + j < room) to[at + j] = next[j];
                     if (n > TAIL_THREADS) break;
                     __syncthreads();
                     h = threadIdx.x < n ? alone[threadIdx.x] : 0u;
@@ -738,7 +741,7 @@ WordBitmaps maps_of(const Plan* p) {
                        static_cast<uint32_t*>(p->reach_stamp.ptr)};
 }
 
-msc_status run_reachability(Plan* p, cudaStream_t s) {
+static msc_status run_levels(Plan* p, cudaStream_t s) {
     const Geom& g = p->g;
     msc_status st;
     const int64_t nrw = int64_t(g.nz) * g.ny * g.W;  // vertex-row words
@@ -765,7 +768,8 @@ msc_status run_reachability(Plan* p, cudaStream_t s) {
     // rerun by sweeps alone
     const bool all = nrw <= TAIL_ROW_WORDS;
     const int64_t sparse = std::max<int64_t>(TAIL_CELLS, nrw / SPARSE_DIV);
-    const int64_t room = all ? 3 * g.nverts : 12 * sparse;
+    int64_t room = all ? 3 * g.nverts : 12 * sparse;
+    if (p->fault_kind == 5) room = std::max<int64_t>(1, std::min<int64_t>(room, p->fault_at));
     if ((st = ensure(p, p->reach_queue, sizeof(uint32_t) * 2 * size_t(room)))) return st;
     PushArgs a{};
     a.g = g;
@@ -811,7 +815,14 @@ msc_status run_reachability(Plan* p, cudaStream_t s) {
         (st = check_cuda(p, cudaMemsetAsync(p->dsum()->push_count, 0, sizeof(p->dsum()->push_count), s), "loop reset")) ||
         (st = check_cuda(p, cudaStreamSynchronize(s), "stream sync")))
         return st;
-    return run_reachability(p, s);
+    return run_levels(p, s);
+}
+
+msc_status run_reachability(Plan* p, cudaStream_t s) {
+    // a field whose levels outgrew the queue says nothing of the next one's; a captured pass does what the
+    // last synchronised one ended with
+    if (!p->capturing) p->reach_sweeps_only = false;
+    return run_levels(p, s);
 }
 
 msc_status run_junctions(Plan* p, cudaStream_t s) {

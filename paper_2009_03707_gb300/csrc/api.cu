@@ -398,6 +398,7 @@ msc_status finish_replay(Plan* p, cudaStream_t s) {
     p->have_gradient = p->have_critical = p->have_extremum = p->have_reach = true;
     p->have_junctions = p->have_trace = p->have_dstar = true;
     ++p->graph_replays;
+    follow_levels(p);
     return MSC_OK;
 }
 

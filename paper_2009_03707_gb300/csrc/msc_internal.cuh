@@ -70,6 +70,8 @@ struct Summary {
     uint32_t push_count[5];           // reachability: the new cells of the pushed levels in hand (reach.cu)
     uint32_t push_cursor;             // reachability: places taken in the queue they start from
     unsigned long long push_iters;    // iterations of the pushed-level loop
+    uint32_t dense;                   // levels that a replayed pass pushed and sweeps should have taken
+    uint32_t pad3;
 };
 
 // ---- the plan ----------------------------------------------------------------------------
@@ -159,7 +161,9 @@ struct Plan {
     int64_t graph_replays = 0;
     int64_t capture_epoch = 0;        // bumped whenever the plan's graph is captured or dropped
     int tail_cluster = 0;             // blocks of the reachability's last-levels cluster (0: not asked yet)
-    int64_t reach_iters = 1;          // sweep iterations of the last synchronised pass (two sweeps each)
+    int64_t reach_iters = 1;          // sweep iterations for the next captured pass (two sweeps each)
+    int64_t reach_captured = 0;       // and those of the captured one (0: a loop, or none)
+    int64_t reach_spare = 0, reach_most = 0;  // replays in a row that left many of them unused; the most these took
     bool reach_sweeps_only = false;   // a level outgrew the push queue in the last synchronised pass
     int grad_variant = -1;            // gradient tile variant (-1: not tuned yet)
 
@@ -272,6 +276,7 @@ msc_status run_junction_dp(Plan* p, cudaStream_t s, uint64_t pool_cap, uint64_t 
 msc_status ensure_reach_maps(Plan* p);  // the buffers of the reachability's bitmaps (reach.cu)
 struct WordBitmaps;
 WordBitmaps maps_of(const Plan* p);
+void follow_levels(Plan* p);  // after a replay: the captured pass's sweeps against what its field took (reach.cu)
 int grid_cap(const Plan* p, int64_t threads, int block, int per_sm = 8);  // grid for a count-bounded loop
 
 }  // namespace msc

@@ -179,10 +179,16 @@ __global__ void reach_start(Summary* sum) {
     sum->loop_flag[3] = 1;  // the sweeps go on
 }
 
+// A replayed pass pushes a level of up to four times the cells at which a level counts as sparse without asking
+// for more sweeps: a sweep iteration that other fields leave unused costs them 5 us, and a level just above
+// the line costs little more pushed than swept (see follow_levels).
+__device__ __forceinline__ uint32_t dense_above(uint32_t sparse) { return 4 * sparse; }
+
 // End of one loop iteration (two sweeps): the non-empty levels found, and the continue decision: while
 // the second sweep still added more than `sparse` cells, up to the iteration cap.  The cells it added
-// are what the pushed levels start from.
-__global__ void reach_decide(Summary* sum, uint32_t sparse, int64_t max_iter, cudaGraphConditionalHandle h, int use_handle) {
+// are what the pushed levels start from.  `last`: there is no further iteration, whatever it added.
+__global__ void reach_decide(Summary* sum, uint32_t sparse, int last, int64_t max_iter, cudaGraphConditionalHandle h,
+                             int use_handle) {
     if (!sum->loop_flag[3]) return;
     const uint32_t c0 = sum->loop_flag[0], c1 = sum->loop_flag[1];
     sum->loop_flag[0] = 0;
@@ -190,6 +196,10 @@ __global__ void reach_decide(Summary* sum, uint32_t sparse, int64_t max_iter, cu
     ++sum->sweep_iters;
     sum->levels += (c0 ? 1 : 0) + (c1 ? 1 : 0);
     bool more = c1 > sparse;
+    if (last) {
+        sum->dense = c1 > dense_above(sparse) ? 1u : 0u;
+        more = false;
+    }
     uint32_t left = more ? 0u : c1;
     if (c1 && int64_t(sum->levels) >= max_iter) {
         atomicOr(&sum->status, uint32_t(ST_ITER));
@@ -356,12 +366,13 @@ __global__ void __launch_bounds__(THREADS) reach_push(PushArgs a, Summary* sum, 
 // End of PUSHES pushed levels: those that were not empty, and whether the last one is still too large
 // for one cluster.  An iteration takes push_count[3] in and leaves its levels in 0, 1, 2 and 4.
 constexpr int PUSHES = 4;
-__global__ void reach_push_decide(Summary* sum, uint32_t few, int64_t max_iter, cudaGraphConditionalHandle h, int use_handle) {
+__global__ void reach_push_decide(Summary* sum, uint32_t few, uint32_t sparse, int64_t max_iter, cudaGraphConditionalHandle h, int use_handle) {
     const uint32_t c[PUSHES] = {sum->push_count[0], sum->push_count[1], sum->push_count[2], sum->push_count[4]};
     uint32_t left = c[PUSHES - 1];
     ++sum->push_iters;
     for (int i = 0; i < PUSHES; ++i) {
         sum->levels += c[i] ? 1 : 0;
+        if (sum->dense && c[i] > dense_above(sparse)) ++sum->dense;
         if ((i & 1) && c[i] && int64_t(sum->levels) >= max_iter) {  // checked at every second level, as by the sweeps
             atomicOr(&sum->status, uint32_t(ST_ITER));
             left = 0;
@@ -380,7 +391,7 @@ __global__ void reach_push_decide(Summary* sum, uint32_t few, int64_t max_iter, 
 // the levels start here, from every cell of the bitmap (the 1-saddles).  The counts live in the first
 // block's shared memory; a cluster barrier ends each level.
 constexpr int TAIL_THREADS = 1024;
-__global__ void __launch_bounds__(TAIL_THREADS, 1) reach_tail(PushArgs a, Summary* sum, int all, int64_t max_iter) {
+__global__ void __launch_bounds__(TAIL_THREADS, 1) reach_tail(PushArgs a, Summary* sum, int all, uint32_t sparse, int64_t max_iter) {
     cg::cluster_group cluster = cg::this_cluster();
     __shared__ uint32_t counts[3], state[2], alone[TAIL_THREADS];
     __shared__ uint64_t state_levels, block_levels;
@@ -419,6 +430,7 @@ __global__ void __launch_bounds__(TAIL_THREADS, 1) reach_tail(PushArgs a, Summar
     // level k reads queue k & 1 and counts its new cells in counts[k % 3]; counts[(k + 1) % 3], last read
     // before level k - 1 began, is cleared for the next level
     uint64_t levels = sum->levels;
+    uint32_t dense = 0;  // levels that sweeps should have taken
     cluster.sync();  // every block has read the counts and the level number
     for (int k = 0; n;) {
         n = min(n, a.cap);
@@ -496,12 +508,16 @@ __global__ void __launch_bounds__(TAIL_THREADS, 1) reach_tail(PushArgs a, Summar
         n = level_n;
         ++k;
         levels += n ? 1 : 0;
+        dense += n > dense_above(sparse) ? 1 : 0;
         if (!(k & 1) && n && int64_t(levels) >= max_iter) {
             if (rank == 0 && threadIdx.x == 0) atomicOr(a.status, ST_ITER);
             n = 0;
         }
     }
-    if (rank == 0 && threadIdx.x == 0) sum->levels = levels;
+    if (rank == 0 && threadIdx.x == 0) {
+        sum->levels = levels;
+        if (sum->dense) sum->dense += dense;
+    }
     cluster.sync();  // no block leaves while others read the first one's counts
 }
 
@@ -660,17 +676,19 @@ struct SweepCtx {
     uint32_t* b;
     uint32_t* stamp;
     uint32_t sparse;
+    int last;
 };
 
 void sweep_body(Plan* p, cudaStream_t s, cudaGraphConditionalHandle h, void* ctx) {
     const SweepCtx& c = *static_cast<SweepCtx*>(ctx);
     reach_sweep<<<c.grid, THREADS, 0, s>>>(p->g, c.masks, c.a, c.b, c.stamp, p->dsum(), 0, &p->dsum()->loop_flag[0]);
     reach_sweep<<<c.grid, THREADS, 0, s>>>(p->g, c.masks, c.b, c.a, c.stamp, p->dsum(), 1, &p->dsum()->loop_flag[1]);
-    reach_decide<<<1, 1, 0, s>>>(p->dsum(), c.sparse, p->opts.max_iterations, h, h != 0);
+    reach_decide<<<1, 1, 0, s>>>(p->dsum(), c.sparse, c.last, p->opts.max_iterations, h, h != 0);
 }
 
 struct PushCtx {
     int grid;
+    uint32_t sparse;
     PushArgs a;
 };
 
@@ -678,11 +696,11 @@ void push_body(Plan* p, cudaStream_t s, cudaGraphConditionalHandle h, void* ctx)
     const PushCtx& c = *static_cast<PushCtx*>(ctx);
     for (int i = 0; i < PUSHES; ++i)
         reach_push<<<c.grid, THREADS, 0, s>>>(c.a, p->dsum(), i & 1, i == 0 ? 3 : i - 1, i == PUSHES - 1 ? 4 : i);
-    reach_push_decide<<<1, 1, 0, s>>>(p->dsum(), TAIL_CELLS, p->opts.max_iterations, h, h != 0);
+    reach_push_decide<<<1, 1, 0, s>>>(p->dsum(), TAIL_CELLS, c.sparse, p->opts.max_iterations, h, h != 0);
 }
 
 // One cluster over as many blocks as this device can schedule together.
-msc_status launch_tail(Plan* p, cudaStream_t s, const PushArgs& a, int all) {
+msc_status launch_tail(Plan* p, cudaStream_t s, const PushArgs& a, int all, uint32_t sparse) {
     msc_status st;
     if (!p->tail_cluster) {
         if ((st = check_cuda(p, cudaFuncSetAttribute(reach_tail, cudaFuncAttributeNonPortableClusterSizeAllowed, 1),
@@ -718,7 +736,7 @@ msc_status launch_tail(Plan* p, cudaStream_t s, const PushArgs& a, int all) {
     cfg.attrs = &at;
     cfg.numAttrs = 1;
     launched(p);
-    return check_cuda(p, cudaLaunchKernelEx(&cfg, reach_tail, a, p->dsum(), all, p->opts.max_iterations), "reach_tail launch");
+    return check_cuda(p, cudaLaunchKernelEx(&cfg, reach_tail, a, p->dsum(), all, sparse, p->opts.max_iterations), "reach_tail launch");
 }
 
 }  // namespace
@@ -761,7 +779,8 @@ static msc_status run_levels(Plan* p, cudaStream_t s) {
     // longer CTAs would cost little alone but leave long tails when other passes share the device.
     const int64_t tiles = (nrw + THREADS - 1) / THREADS;
     const int64_t sweep_ctas = std::min<int64_t>(tiles, std::max<int64_t>(int64_t(std::max(1, p->num_sms)) * 4, (tiles + 3) / 4));
-    SweepCtx ctx{dim3(unsigned(std::max<int64_t>(1, sweep_ctas)), 1), masks, A, B, stamp, 0};
+    SweepCtx ctx{dim3(unsigned(std::max<int64_t>(1, sweep_ctas)), 1), masks, A, B, stamp, 0, 0};
+    if (p->capturing) p->reach_captured = 0;
     if (p->reach_sweeps_only) return run_loop(p, s, 1, 3, sweep_body, &ctx);
     // the pushed levels.  A small grid's queues hold every 1-cell; a large one's twelve times the level
     // they start from (a level of a sparse front hardly grows), and a pass that needs more asks for a
@@ -786,9 +805,10 @@ static msc_status run_levels(Plan* p, cudaStream_t s) {
         } else {
             // as many iterations as the last synchronised pass took, one after another (a conditional
             // node costs 12 us an iteration): a field that needs fewer skips the rest, one that needs
-            // more pushes a larger level
+            // more pushes a larger level (see follow_levels)
+            p->reach_captured = p->reach_iters;
             for (int64_t i = 0; i < p->reach_iters; ++i) {
-                if (i + 1 == p->reach_iters) ctx.sparse = 0xFFFFFFFFu;
+                ctx.last = i + 1 == p->reach_iters;
                 sweep_body(p, s, 0, &ctx);
                 launched(p, 3);
             }
@@ -798,11 +818,11 @@ static msc_status run_levels(Plan* p, cudaStream_t s) {
         reach_frontier<<<grid_for(p, nrw), THREADS, 0, s>>>(a, A, B, &sum->push_count[3], &sum->push_cursor);
         launched(p);
         if (sparse > TAIL_CELLS) {
-            PushCtx pc{std::max(1, p->num_sms) * 8, a};
+            PushCtx pc{std::max(1, p->num_sms) * 8, ctx.sparse, a};
             if ((st = run_loop(p, s, 3, PUSHES + 1, push_body, &pc))) return st;
         }
     }
-    if ((st = launch_tail(p, s, a, all ? 1 : 0))) return st;
+    if ((st = launch_tail(p, s, a, all ? 1 : 0, uint32_t(sparse)))) return st;
     if (p->capturing) return MSC_OK;
     // a synchronised pass whose queue was full (a replayed one comes here through its rerun)
     if ((st = read_summary(p, s))) return st;
@@ -823,6 +843,29 @@ msc_status run_reachability(Plan* p, cudaStream_t s) {
     // last synchronised one ended with
     if (!p->capturing) p->reach_sweeps_only = false;
     return run_levels(p, s);
+}
+
+// A replayed pass sweeps as often as it was captured to, so the next one is captured for the field of this
+// one if that had levels for sweeps that it had to push, or if MANY replays in a row left more than SPARE
+// iterations unused.  Fields in turn do not make a plan capture again and again (0.25 ms each): the number grows
+// at once, and only many replays together make it fall.  Reachability stage of a GRF that takes three
+// iterations, captured with two: 140^3 (the levels go to one cluster) 171 us, 85 once captured again; 152^3 119
+// and 110, 256^3 230 and 207.  An unused iteration takes 5 us.
+void follow_levels(Plan* p) {
+    constexpr int64_t SPARE = 1, MANY = 64;
+    if (!p->reach_captured) return;
+    const int64_t took = int64_t(p->hsum->sweep_iters);
+    if (p->hsum->dense) {  // the handed-over level and dense - 1 after it; an iteration ends at every second level
+        p->reach_iters = p->reach_captured + 1 + (int64_t(p->hsum->dense) - 1) / 2;
+    } else {
+        const bool spare = p->reach_captured - took > SPARE;
+        p->reach_spare = spare ? p->reach_spare + 1 : 0;
+        p->reach_most = spare ? std::max(p->reach_most, took) : 0;
+        if (p->reach_spare < MANY) return;
+        p->reach_iters = std::max<int64_t>(1, p->reach_most);
+    }
+    p->reach_spare = p->reach_most = 0;
+    destroy_graph(p);
 }
 
 msc_status run_junctions(Plan* p, cudaStream_t s) {

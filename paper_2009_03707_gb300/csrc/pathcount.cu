@@ -1084,7 +1084,8 @@ msc_status run_path_count(Plan* p, cudaStream_t s) {
         int left_list = 1;
         u64* left_ctr = ctr + C_DEFER2;
         if (first_tier == 0) {
-            if (n1cap > GROUP_FIRST || p->opts.path_count_tier < 0) {
+            // by the last pass's count: a captured pass's capacity lies a quarter and 1024 above it
+            if (p->counts[1] > GROUP_FIRST || p->opts.path_count_tier < 0) {
                 if ((st = launch(0, nullptr, all_rows, lists[0], ctr + C_DEFER0, 0, false))) return st;
                 if ((st = launch(3, lists[0], ctr + C_DEFER0, lists[1], ctr + C_DEFER1, 0, false))) return st;
             } else if ((st = launch(3, nullptr, all_rows, lists[1], ctr + C_DEFER1, 0, false))) {

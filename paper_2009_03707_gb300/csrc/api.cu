@@ -154,8 +154,9 @@ msc_status run_loop(Plan* p, cudaStream_t s, int which, int body_launches,
                       "capture dependencies");
 }
 
-// MSC_FAULT = alloc@k | capture@k | queue@n | timeout | overflow (the k-th growth of a buffer or the k-th capture
-// fails; the reachability's queues have room for n cells): host-side fault injection for tests.
+// MSC_FAULT = alloc@k | capture@k | queue@n | rows@n | timeout | overflow (the k-th growth of a buffer or the k-th
+// capture fails; the reachability's queues have room for n cells; the simplification's row pools start with n
+// entries beyond the complex): host-side fault injection for tests.
 void read_fault(Plan* p) {
     const char* f = std::getenv("MSC_FAULT");
     if (!f) return;
@@ -168,6 +169,9 @@ void read_fault(Plan* p) {
     } else if (!std::strncmp(f, "queue@", 6)) {
         p->fault_kind = 5;
         p->fault_at = std::atoll(f + 6);
+    } else if (!std::strncmp(f, "rows@", 5)) {
+        p->fault_kind = 6;
+        p->fault_at = std::atoll(f + 5);
     } else if (!std::strcmp(f, "timeout")) {
         p->fault_kind = 2;
     } else if (!std::strcmp(f, "overflow")) {

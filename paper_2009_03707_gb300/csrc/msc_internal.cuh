@@ -200,7 +200,8 @@ struct Plan {
     cudaStream_t pending_stream = nullptr;
     // host-side fault injection (MSC_FAULT, read at plan creation; tests only): the failure is
     // made on the host -- a faked allocation failure, or a status bit raised as a kernel would
-    int fault_kind = 0;  // 0 none, 1 alloc, 2 timeout (reachability), 3 overflow (path count), 4 capture, 5 a small queue (reachability)
+    int fault_kind = 0;  // 0 none, 1 alloc, 2 timeout (reachability), 3 overflow (path count), 4 capture, 5 a small queue (reachability),
+                         // 6 small row pools (simplification)
     int64_t fault_at = 0, fault_calls = 0;
 };
 

@@ -856,7 +856,7 @@ msc_status run_simplify(Plan* p, const float* d_field, double threshold, cudaStr
     };
     u64 cap[2];
     for (int b = 0; b < 2; ++b) {
-        cap[b] = u64(nnz0) + u64(nnz0) / 4 + 256;
+        cap[b] = u64(nnz0) + (p->fault_kind == 6 ? u64(p->fault_at) : u64(nnz0) / 4 + 256);
         if ((st = pool(b, cap[b]))) return st;
     }
     char* w = static_cast<char*>(p->simp_node.ptr);

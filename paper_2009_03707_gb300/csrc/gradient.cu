@@ -108,7 +108,7 @@ __global__ void __launch_bounds__(THREADS, 65536 / (64 * THREADS)) gradient_kern
         const int gx = x0 - 1 + fx, gy = y0 - 1 + fy, gz = z0 - 1 + fz;
         const bool in = gx >= 0 && gy >= 0 && gz >= 0 && gx < g.nx && gy < g.ny && gz < g.nz;
         saw_nan |= in && isnan(v[k]);
-        sh.fkey[fz][fy][fx] = in ? star::order_key_of_bits(__float_as_uint(v[k])) : OUTSIDE_KEY;
+        sh.fkey[fz][fy][fx] = in ? star::order_key_of(v[k]) : OUTSIDE_KEY;
     }
     if (saw_nan) atomicOr(status, ST_NAN);
     __syncthreads();

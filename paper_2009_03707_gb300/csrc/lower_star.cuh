@@ -42,10 +42,17 @@
 #define MSC_FFS(x) __ffs(x)
 #define MSC_POPC(x) __popc(x)
 #define MSC_UMIN(a, b) min(a, b)
+#define MSC_FLOAT_BITS(f) __float_as_uint(f)
 #else
 #define MSC_FFS(x) __builtin_ffs(int(x))
 #define MSC_POPC(x) __builtin_popcount(x)
 #define MSC_UMIN(a, b) ((a) < (b) ? (a) : (b))
+#define MSC_FLOAT_BITS(f) msc_float_bits(f)
+inline uint32_t msc_float_bits(float f) {
+    uint32_t u;
+    __builtin_memcpy(&u, &f, sizeof(u));
+    return u;
+}
 #endif
 
 namespace msc {
@@ -105,14 +112,14 @@ __host__ __device__ inline uint32_t cell_vertices(int p) {
     return xs & ys & zs & ~(1u << CENTER);
 }
 
-// Monotone map of a float's bits to uint32 (IEEE order; -0 and +0 map to the same key).  Every NaN above
-// infinity gets one key, just above infinity's: a field with a NaN is rejected, but the kernel has run on it
-// by then, and a NaN's own bits reach up to the key of an off-grid vertex and to the padding words of
+// Monotone map float -> uint32 (IEEE order; -0 and +0 map to the same key: the sum with +0 is +0 for both).
+// No NaN's key exceeds NAN_KEY, just above infinity's: a field with a NaN is rejected, but the kernel has run on
+// it by then, and a NaN's own bits reach up to the key of an off-grid vertex and to the padding words of
 // rank_cell_keys, which have to stay above every key of the grid.
 constexpr uint32_t NAN_KEY = 0xFF800001u;
-__host__ __device__ __forceinline__ uint32_t order_key_of_bits(uint32_t u) {
-    if ((u & 0x7FFFFFFFu) == 0) u = 0;
-    return (u & 0x80000000u) ? ~u : MSC_UMIN(u | 0x80000000u, NAN_KEY);
+__host__ __device__ __forceinline__ uint32_t order_key_of(float f) {
+    const uint32_t u = MSC_FLOAT_BITS(f + 0.0f);
+    return MSC_UMIN(u ^ (uint32_t(int32_t(u) >> 31) | 0x80000000u), NAN_KEY);
 }
 
 // Per-position masks, tabulated once per CTA (shared memory on the device): a 27-entry table of

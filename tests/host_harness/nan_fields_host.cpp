@@ -19,7 +19,8 @@ int main(int argc, char** argv) {
     int64_t d[3];
     if (!in || std::fread(d, sizeof(int64_t), 3, in) != 3) return 2;
     const int nx = int(d[0]), ny = int(d[1]), nz = int(d[2]);
-    std::vector<uint32_t> field(size_t(nx) * ny * nz), words(field.size(), 0u);
+    std::vector<float> field(size_t(nx) * ny * nz);
+    std::vector<uint32_t> words(field.size(), 0u);
     if (std::fread(field.data(), 4, field.size(), in) != field.size()) return 2;
     std::fclose(in);
     static Tables T;
@@ -31,7 +32,7 @@ int main(int argc, char** argv) {
                 for (int p = 0; p < 27; p++) {
                     const int X = x + pdx(p), Y = y + pdy(p), Z = z + pdz(p);
                     const bool out = X < 0 || Y < 0 || Z < 0 || X >= nx || Y >= ny || Z >= nz;
-                    k[p] = out ? 0xFFFFFFFFu : order_key_of_bits(field[size_t(X) + nx * (size_t(Y) + ny * size_t(Z))]);
+                    k[p] = out ? 0xFFFFFFFFu : order_key_of(field[size_t(X) + nx * (size_t(Y) + ny * size_t(Z))]);
                 }
                 auto emit = [&](int p, uint32_t code) {
                     const int dx = pdx(p), dy = pdy(p), dz = pdz(p);

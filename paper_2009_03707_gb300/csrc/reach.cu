@@ -26,8 +26,9 @@
 //    the same.  Large grids push with the whole device while a level is large; the last levels --
 //    and on a small grid all of them -- run in one kernel of one thread-block cluster, whose
 //    hardware barrier between levels costs far less than a kernel boundary.
-//    Reachability stage: 512^3 blobs 15.9 -> 4.9 ms, 256^3 GRF 0.395 -> 0.299, 61 x 75 x 49 GRF 0.102 ->
-//    0.072, 32^3 lattice (19 levels) 0.127 -> 0.072.
+//    Reachability stage of a replayed pass, against sweeps for every level: 512^3 blobs 15.9 -> 3.8 ms,
+//    256^3 GRF 0.395 -> 0.200, 61 x 75 x 49 GRF 0.102 -> 0.064, 32^3 lattice (19 levels) 0.127 -> 0.061 (0.74
+//    and 0.095 ms of the first two were the bitmaps, which a replay makes in the gradient stage since).
 //
 // Sec. 3.3 / Sec. 3.5 "Gradient path counting": a junction is a reachable 1-cell that is not a
 // 1-saddle and has out-degree > 1.  One warp per bitmap word (a lane per 1-cell) evaluates the
@@ -658,9 +659,11 @@ int grid_for(const Plan* p, int64_t threads) {
     return int(std::max<int64_t>(1, std::min(want, cap)));
 }
 
-// Grids of at most this many row words push every level in one cluster: 0.072 ms against 0.127 by
-// sweeps on a 1024-word lattice, but 0.164 against 0.072 (two sweep iterations, then the cluster) on a
-// 7350-word GRF, whose first levels have 100 thousand cells.
+// Grids of at most this many row words push every level in one cluster.  What decides is the levels' sizes,
+// which the grid only bounds: against sweeps first, then the cluster, it is even on smooth fields of any of
+// these sizes and on rough ones up to 1024 row words (24^3 white noise 37 us either way, 32^3 GRF 49), and
+// slower on rough ones near the line (2040 words: GRF k^-2 61 against 49 us, white noise 62-72 against 39-47;
+// 70-82 by sweeps alone); a 7350-word GRF, whose first levels have 100 thousand cells, took 164 against 72.
 constexpr int64_t TAIL_ROW_WORDS = 2048;
 // A level of at most this many new cells is left to one cluster (two cells a thread; 128 thousand, eight
 // a thread, took 1.5 ms of the 512^3 blob field's levels that the whole device pushes in 0.6 ms) ...

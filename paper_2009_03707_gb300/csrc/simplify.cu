@@ -30,8 +30,10 @@
 // Four launches a round, their counts on the device; the host looks once per BATCH rounds.  At the
 // end one gather makes the CSR, and one stable sort by round puts the cancellations in log order.
 // 256^3 GRF (6.0 M nodes, 40 M entries, 317 rounds, threshold 5 % of the range): 370 ms with every
-// round sweeping all nodes and rewriting the whole CSR (1.1 ms a round), 66 ms now: looks 28, updates 14,
-// the list 11, cancellations 6.
+// round sweeping all nodes and rewriting the whole CSR (1.1 ms a round), 67 ms now: looks 27, updates 14,
+// the list 11, cancellations 6, gathers 2.  The price is memory: 188 B a node (161 of them in simp_node, 40 the
+// two lists) and two row pools of 1.25 x 12 B an entry, 2.7 GB there, where the sweeps took 117 B and two copies
+// of the rows, 1.9 GB.
 #include <cooperative_groups.h>
 
 #include "radix.cuh"
@@ -463,9 +465,11 @@ __device__ __forceinline__ void look_at_arcs(const SimpArgs& a, RoundCount* out,
         }
     }
 }
-// Many looks are bound by how many are in flight (8 lanes each), few by how long the longest takes (a
-// whole warp each): late rounds of the 256^3 GRF have some 2500 looks of up to 1850 entries (all looks:
-// 40, 37 and 35 ms with the line at 16, 32 and 64 thousand).
+// Few looks are bound by how long the longest takes, so they get a whole warp each: late rounds of the 256^3
+// GRF have some 2500 looks of up to 1850 entries.  Where there are many, eight lanes each were meant to keep
+// more in flight; the measured gain is gone.  Whole call with the line at 16, 64, 128 and 256 thousand: 73.4,
+// 66.9, 66.2, 66.1 ms; a warp for every look 66.1; sixteen lanes above the line 65.9, four 68.5; sixteen
+// lanes below it 72.7.
 constexpr unsigned int WIDE_LOOKS = 65536;
 __global__ void __launch_bounds__(THREADS) simp_look(SimpArgs a, int slot) {
     if (a.state->halted) return;

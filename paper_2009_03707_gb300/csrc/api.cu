@@ -171,7 +171,7 @@ void read_fault(Plan* p) {
         p->fault_at = std::atoll(f + 6);
     } else if (!std::strncmp(f, "rows@", 5)) {
         p->fault_kind = 6;
-        p->fault_at = std::atoll(f + 5);
+        p->fault_at = std::max<int64_t>(0, std::atoll(f + 5));
     } else if (!std::strcmp(f, "timeout")) {
         p->fault_kind = 2;
     } else if (!std::strcmp(f, "overflow")) {

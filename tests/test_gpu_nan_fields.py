@@ -6,6 +6,7 @@ import numpy as np
 import pytest
 import torch
 
+import oracle
 from tests.gpu_util import dims_of, gpu_field, msc, to_np
 from tests.test_kernel_core_nan import _masks
 
@@ -42,3 +43,15 @@ def test_nan_regions_are_rejected(mask, bits):
         m.msc_gradient_critical_static(bad, words, cells, [n] * 4)
     assert e.value.status == 2
     assert m.msc_gradient_critical_static(field, words, cells, [n] * 4) == m.msc_critical(alone)[0]
+
+
+def test_numbers_of_every_size_keep_their_words():
+    """Both zeros, denormals, the largest numbers and infinities, many of them equal, against the oracle."""
+    m = msc()
+    rng = np.random.default_rng(12)
+    bits = np.array([0, 1, 2, 0x7FFFFF, 0x800000, 0x3F800000, 0x7F7FFFFF, 0x7F800000], np.uint32)
+    f = (rng.choice(bits, (13, 21, 35)) | (rng.integers(0, 2, (13, 21, 35), dtype=np.uint32) << 31)).view(np.float32)
+    plan = m.Plan(dims_of(f))
+    m.msc_gradient(plan, gpu_field(f))
+    m.msc_critical(plan)
+    assert np.array_equal(to_np(m.msc_gradient_words(plan)), oracle.pack(dims_of(f), oracle.gradient(f)))
